@@ -93,8 +93,6 @@ struct ModelRows {
     uint8_t *lod;       // may be NULL
 };
 
-__device__ constexpr int kRowLen[5] = {3, 3, 4, 1, 48};
-
 struct ScatterArgs {
     ModelRows src, dst;
     long long n;
@@ -108,8 +106,18 @@ struct ScatterArgs {
     int max_level;
     unsigned long long *lb_status;
     long long *n_out;     // device
+    // the output rows, in order: source Gaussian (the first list_n in list0, the
+    // rest, of density control, in list1) and how the row is made (RowHow)
+    uint32_t *list0, *list1;
+    long long list_n;
+    uint8_t *how;
     DevCounters *ctr;
 };
+
+// How an output row is made from its source: a copy with its moments, a copy
+// whose moments start from zero (a clone), a split child (its mean and scales
+// written already, moments from zero), or not written (it lies past dst_cap).
+enum RowHow { kRowCopy = 0, kRowClone = 1, kRowChild = 2, kRowNone = 3 };
 
 // 0 removed, 1 kept, 2 cloned, 3 split: FP32 quantities formed as the oracle
 // forms them (its decision instance mirrors these operations).
@@ -124,22 +132,15 @@ __device__ __forceinline__ int densify_kind(const ScatterArgs &a, long long i)
     return fmaxf(ls[0], fmaxf(ls[1], ls[2])) <= a.log_dense ? 2 : 3;
 }
 
-__device__ __forceinline__ void copy_row(const ModelRows &s, long long i, const ModelRows &d, long long o, bool moments)
+__device__ __forceinline__ void put_row(const ScatterArgs &a, long long o, long long i, RowHow how)
 {
-#pragma unroll
-    for (int k = 0; k < 5; k++) {
-        const int L = kRowLen[k];
-        for (int e = 0; e < L; e++) d.p[k][o * L + e] = s.p[k][i * L + e];
-        if (d.m[k]) for (int e = 0; e < L; e++) d.m[k][o * L + e] = moments && s.m[k] ? s.m[k][i * L + e] : 0.f;
-        if (d.v[k]) for (int e = 0; e < L; e++) d.v[k][o * L + e] = moments && s.v[k] ? s.v[k][i * L + e] : 0.f;
-    }
-    if (d.lod) d.lod[o] = s.lod ? s.lod[i] : 0;
+    (o < a.list_n ? a.list0 : a.list1 - a.list_n)[o] = (uint32_t)i;
+    a.how[o] = (uint8_t)how;
 }
 
-// One split child: mu + R(q) (s * z), log-scale - log(1.6), next finer level.
+// The mean and scales of one split child: mu + R(q) (s * z), log-scale - log(1.6).
 __device__ __forceinline__ void write_child(const ScatterArgs &a, long long i, long long o, int c)
 {
-    copy_row(a.src, i, a.dst, o, false);
     const float *q = a.src.p[2] + 4 * i;
     const float qn = sqrtf(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
     const float w = q[0] / qn, x = q[1] / qn, y = q[2] / qn, z = q[3] / qn;
@@ -153,14 +154,12 @@ __device__ __forceinline__ void write_child(const ScatterArgs &a, long long i, l
         a.dst.p[0][3 * o + r] = a.src.p[0][3 * i + r] + (R[r][0] * l[0] + R[r][1] * l[1] + R[r][2] * l[2]);
         a.dst.p[1][3 * o + r] = ls[r] - a.log_shrink;
     }
-    if (a.dst.lod) {
-        const int lv = (a.src.lod ? (int)a.src.lod[i] : 0) + 1;
-        a.dst.lod[o] = (uint8_t)(lv < a.max_level ? lv : a.max_level);
-    }
 }
 
-// Ticket-ordered blocks of 256 Gaussians: each block counts its outputs,
-// finds its offset by decoupled look-back and writes them in parent order.
+// The list of output rows.  Ticket-ordered blocks of 256 Gaussians: each block
+// counts its outputs, finds its offset by decoupled look-back and writes its
+// rows' sources in parent order, with the levels and the split children's mean
+// and scales; model_rows_kernel then copies the rows.
 __global__ void __launch_bounds__(256) model_scatter_kernel(ScatterArgs a)
 {
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
@@ -187,16 +186,115 @@ __global__ void __launch_bounds__(256) model_scatter_kernel(ScatterArgs a)
     if (cnt == 0) return;
     if ((long long)(o + cnt) > a.dst_cap) {
         set_error(a.ctr, GS_ERR_CAPACITY, kSiteModel);
+        if ((long long)o < a.dst_cap) put_row(a, (long long)o, i, kRowNone); // the first of two rows
         return;
     }
-    if (kind == 1) copy_row(a.src, i, a.dst, (long long)o, true);
-    else if (kind == 2) {
-        copy_row(a.src, i, a.dst, (long long)o, true);
-        copy_row(a.src, i, a.dst, (long long)o + 1, false);
+    const long long r = (long long)o;
+    if (kind == 3) {
+        for (int c = 0; c < 2; c++) {
+            put_row(a, r + c, i, kRowChild);
+            write_child(a, i, r + c, c);
+        }
     } else {
-        write_child(a, i, (long long)o, 0);
-        write_child(a, i, (long long)o + 1, 1);
+        put_row(a, r, i, kRowCopy);
+        if (kind == 2) put_row(a, r + 1, i, kRowClone);
     }
+    if (a.dst.lod) {
+        int lv = a.src.lod ? (int)a.src.lod[i] : 0;
+        if (kind == 3) lv = min(lv + 1, a.max_level); // the next finer level
+        a.dst.lod[r] = (uint8_t)lv;
+        if (cnt == 2) a.dst.lod[r + 1] = (uint8_t)lv;
+    }
+}
+
+// One array of the model, LEN floats per row: output elements in order, four
+// per thread (a float4 where the output is 16-byte aligned, and of one source
+// row where LEN is a multiple of four and the source is aligned too).
+// moment: rows other than plain copies start from zero (all rows without a
+// source array); geom: the split children's values are in place already.  A
+// list entry left unset by a look-back that gave up is not followed (i < n).
+template <int LEN>
+__device__ __forceinline__ void copy_rows(const ScatterArgs &a, const float *__restrict__ src, float *__restrict__ dst,
+                                          long long rows, bool moment, bool geom)
+{
+    if (!dst) return;
+    const bool vdst = ((uintptr_t)dst & 15u) == 0, vsrc = LEN % 4 == 0 && src && ((uintptr_t)src & 15u) == 0;
+    const unsigned long long total = (unsigned long long)rows * LEN, chunks = (total + 3) / 4;
+    const unsigned long long stride = gridDim.x * 256ull;
+#pragma unroll 4 // the loads of four chunks in flight
+    for (unsigned long long c = blockIdx.x * 256ull + threadIdx.x; c < chunks; c += stride) {
+        const unsigned long long e0 = 4 * c;
+        float v[4] = {0.f, 0.f, 0.f, 0.f};
+        bool put = true; // all four elements are written
+        if (LEN % 4 == 0) {
+            const long long o = (long long)(e0 / LEN);
+            const int how = a.how[o];
+            const long long i = (o < a.list_n ? a.list0 : a.list1 - a.list_n)[o];
+            put = i < a.n && how != kRowNone && !(geom && how == kRowChild);
+            if (put && src && !(moment && how != kRowCopy)) {
+                const float *s = src + i * LEN + (long long)(e0 % LEN);
+                if (vsrc) {
+                    const float4 q = __ldcs(reinterpret_cast<const float4 *>(s));
+                    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+                } else {
+#pragma unroll
+                    for (int u = 0; u < 4; u++) v[u] = s[u];
+                }
+            }
+            if (!put) continue;
+            if (vdst) __stcs(reinterpret_cast<float4 *>(dst + e0), make_float4(v[0], v[1], v[2], v[3]));
+            else {
+#pragma unroll
+                for (int u = 0; u < 4; u++) dst[e0 + u] = v[u];
+            }
+        } else {
+            bool w[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const unsigned long long e = e0 + u;
+                w[u] = e < total;
+                if (w[u]) {
+                    const long long o = (long long)(e / LEN);
+                    const int how = a.how[o];
+                    const long long i = (o < a.list_n ? a.list0 : a.list1 - a.list_n)[o];
+                    w[u] = i < a.n && how != kRowNone && !(geom && how == kRowChild);
+                    if (w[u] && src && !(moment && how != kRowCopy)) v[u] = src[i * LEN + (long long)(e % LEN)];
+                }
+                put = put && w[u];
+            }
+            if (put && vdst) __stcs(reinterpret_cast<float4 *>(dst + e0), make_float4(v[0], v[1], v[2], v[3]));
+            else {
+#pragma unroll
+                for (int u = 0; u < 4; u++)
+                    if (w[u]) dst[e0 + u] = v[u];
+            }
+        }
+    }
+}
+
+// The rows of the list, array by array: consecutive threads write consecutive
+// output elements and read consecutive elements of a source row, so both
+// sides move whole sectors.  Bound by HBM (708 bytes read and written per row
+// of a model with moments).
+__global__ void __launch_bounds__(256, 4) model_rows_kernel(ScatterArgs a)
+{
+    griddep_wait(); // programmatic dependent launch: the previous kernel is complete
+    const long long rows = min(*a.n_out, a.dst_cap);
+    copy_rows<48>(a, a.src.p[4], a.dst.p[4], rows, false, false);
+    copy_rows<48>(a, a.src.m[4], a.dst.m[4], rows, true, false);
+    copy_rows<48>(a, a.src.v[4], a.dst.v[4], rows, true, false);
+    copy_rows<4>(a, a.src.p[2], a.dst.p[2], rows, false, false);
+    copy_rows<4>(a, a.src.m[2], a.dst.m[2], rows, true, false);
+    copy_rows<4>(a, a.src.v[2], a.dst.v[2], rows, true, false);
+#pragma unroll 1
+    for (int k = 0; k < 2; k++) { // mean, log-scale
+        copy_rows<3>(a, a.src.p[k], a.dst.p[k], rows, false, true);
+        copy_rows<3>(a, a.src.m[k], a.dst.m[k], rows, true, false);
+        copy_rows<3>(a, a.src.v[k], a.dst.v[k], rows, true, false);
+    }
+    copy_rows<1>(a, a.src.p[3], a.dst.p[3], rows, false, false);
+    copy_rows<1>(a, a.src.m[3], a.dst.m[3], rows, true, false);
+    copy_rows<1>(a, a.src.v[3], a.dst.v[3], rows, true, false);
 }
 
 // Views in which each Gaussian has a record (+= per Gaussian; records of a
@@ -267,7 +365,15 @@ cudaError_t launch_model_scatter(gs_workspace *ws, cudaStream_t st, ScatterArgs 
     a.lb_status = ws->mlb;
     a.ctr = ws->mctr;
     if (blocks == 0) return cudaSuccess;
+    // the row list in the sort scratch of the selections (their keys and values
+    // are read by now): up to two rows per Gaussian, one byte each for how
+    a.list0 = ws->mkey[0];
+    a.list1 = ws->mkey[1];
+    a.list_n = ws->cap.max_gaussians;
+    a.how = reinterpret_cast<uint8_t *>(ws->mval[0]);
     launch_pdl(model_scatter_kernel, (unsigned)blocks, 256, 0, st, a);
+    note_launch();
+    launch_pdl(model_rows_kernel, 8u * (unsigned)ws->sm_count, 256, 0, st, a);
     note_launch();
     return cudaGetLastError();
 }
