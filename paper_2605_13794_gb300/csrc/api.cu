@@ -46,13 +46,13 @@ struct Layout {
 };
 
 struct Offsets {
-    size_t cand_g, cand_mask, gate_g, gate_mask, rec_first, cgrad, rec_g, rec_cam, rd0, rd1, rd2, rect, tt, inst_off, clampm, rgrad, dkey, tile_cnt, tile_cur, tile_last;
+    size_t cand_g, cand_mask, gate_cnt, gate_g, gate_mask, rec_first, cgrad, rec_g, rec_cam, rd0, rd1, rd2, rect, tt, inst_off, clampm, rgrad, dkey, tile_cnt, tile_cur, tile_last;
     size_t tkey0, tkey1, tval0, tval1, slots, imp_slots, ranges, n_contrib, T_final, imp_w, imp_a, sel_cum, sel_bsum;
-    size_t selk0, selk1, selv0, selv1, loss_maps, loss_partial, lb_status, rx_status, red_partial,
+    size_t selk0, selk1, selv0, selv1, loss_maps, loss_partial, lb_status, bin_lb, rx_status, red_partial,
         ctr, d_cams, d_adam_step, d_adam_coef;
     size_t mkey0, mkey1, mval0, mval1, mcum, mbsum, mrx_status, mlb, mhist, mctr;
     size_t total;
-    size_t lb_words, rx_words, red_words, loss_partial_words;
+    size_t lb_words, bin_lb_words, rx_words, red_words, loss_partial_words;
 };
 
 Offsets plan(const gs_capacity &c)
@@ -63,6 +63,7 @@ Offsets plan(const gs_capacity &c)
     const size_t T = (size_t)c.max_tiles, P = (size_t)c.max_pixels;
     o.cand_g = L.take<uint32_t>(N);
     o.cand_mask = L.take<unsigned long long>(N);
+    o.gate_cnt = L.take<uint16_t>(N / 128 + 1);
     o.gate_g = L.take<uint32_t>(N);
     o.gate_mask = L.take<unsigned long long>(N);
     o.rec_first = L.take<uint32_t>(N);
@@ -102,12 +103,13 @@ Offsets plan(const gs_capacity &c)
     o.loss_maps = L.take<float>(fwd_only ? 0 : P * 3 * 3); // per pixel and channel: F0, F1, F2 (planar)
     o.loss_partial_words = fwd_only ? 0 : 2 * 3 * (P / 1024 + 65536);
     o.loss_partial = L.take<float>(o.loss_partial_words);
-    // look-back words: one per chunk of the smallest chunked pass (the
-    // projection's candidates) plus the ticket, and the binning's two regions
-    // (records of its count pass, tiles of its tile scan)
-    const size_t nb = (N > R ? N : R) / 64 + 2;
-    o.lb_words = nb + 1 + T / 1024 + 4;
+    // look-back words of the preprocess: one per 128 candidates of the
+    // projection, one per 8192 Gaussians of the gather, and their tickets
+    o.lb_words = N / 128 + N / 8192 + 8;
     o.lb_status = L.take<unsigned long long>(o.lb_words);
+    // ... of the binning: 128 records of its count pass, 1024 tiles of its scan
+    o.bin_lb_words = R / 128 + T / 1024 + 8;
+    o.bin_lb = L.take<unsigned long long>(o.bin_lb_words);
     const size_t items = (R > I ? R : I);
     // the histograms, then the look-back state of up to four passes, for the
     // smallest (1024-key) blocks
@@ -264,6 +266,7 @@ int gs_workspace_create(const gs_capacity *cap, gs_workspace **out)
     char *b = (char *)ws->base;
     ws->cand_g = (uint32_t *)(b + o.cand_g);
     ws->cand_mask = (unsigned long long *)(b + o.cand_mask);
+    ws->gate_cnt = (uint16_t *)(b + o.gate_cnt);
     ws->gate_g = (uint32_t *)(b + o.gate_g);
     ws->gate_mask = (unsigned long long *)(b + o.gate_mask);
     ws->rec_first = (uint32_t *)(b + o.rec_first);
@@ -300,6 +303,8 @@ int gs_workspace_create(const gs_capacity *cap, gs_workspace **out)
     ws->loss_partial_words = o.loss_partial_words;
     ws->lb_status = (unsigned long long *)(b + o.lb_status);
     ws->lb_words = o.lb_words;
+    ws->bin_lb = (unsigned long long *)(b + o.bin_lb);
+    ws->bin_lb_words = o.bin_lb_words;
     ws->rx_status = (uint32_t *)(b + o.rx_status);
     ws->rx_words = o.rx_words;
     ws->rx_hist = ws->rx_status; // the first kRxHistWords words
@@ -319,6 +324,9 @@ int gs_workspace_create(const gs_capacity *cap, gs_workspace **out)
     ws->mctr = (gs::DevCounters *)(b + o.mctr);
     e = cudaMemset(ws->ctr, 0, sizeof(gs::DevCounters));
     if (e == cudaSuccess) e = cudaMemset(ws->d_cams, 0, sizeof(gs::CamTable));
+    // zero between binnings: every binning leaves them so
+    if (e == cudaSuccess) e = cudaMemset(ws->bin_lb, 0, o.bin_lb_words * sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaMemset(ws->tile_cnt, 0, (size_t)cap->max_tiles * sizeof(uint32_t));
     if (e == cudaSuccess) e = cudaMemset(ws->d_adam_step, 0, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(ws->mctr, 0, sizeof(gs::DevCounters));
     if (e == cudaSuccess) e = cudaMallocHost(&ws->h_stage, gs_workspace::kStageSlots * sizeof(gs::CamTable));
@@ -547,10 +555,8 @@ int gs_bin_sort(gs_workspace *ws, gs_stream stream)
     if (!ws) return fail(GS_ERR_INVALID_ARG, "gs_bin_sort: NULL workspace");
     if (!ws->have_preprocess) return fail(GS_ERR_INVALID_ARG, "gs_bin_sort: no preprocess on this workspace");
     cudaStream_t st = (cudaStream_t)stream;
-    // the instance counters, then tile counts, ranges, scatter and the
-    // per-tile depth sort (the final order: camera, tile, depth bits, record)
-    CK(cudaMemsetAsync(&ws->ctr->n_instances, 0, sizeof(unsigned long long), st), "gs_bin_sort");
-    CK(cudaMemsetAsync(&ws->ctr->instances_needed, 0, sizeof(unsigned long long), st), "gs_bin_sort");
+    // tile counts, ranges, scatter and the per-tile depth sort (the final
+    // order: camera, tile, depth bits, record)
     CK(gs::launch_bin(ws, st), "gs_bin_sort");
     ws->tile_buf = 0;
     ws->have_binning = 1;

@@ -20,6 +20,8 @@
 // The final order of a tile's list is (depth bits, record): depth ties go to
 // the lower record, i.e. the lower Gaussian index.  Counts stay on the
 // device; nothing here synchronises with the host.
+#include <algorithm>
+
 #include "gs_internal.cuh"
 
 namespace gs {
@@ -36,7 +38,7 @@ struct BinArgs {
     const uint16_t *rec_cam;
     const uint32_t *dkey;          // FP32 bits of each record's camera depth
     uint32_t *inst_off;            // first instance of each record (record order)
-    uint32_t *tile_cnt;            // [tiles] instances per tile (zeroed before the count)
+    uint32_t *tile_cnt;            // [tiles] instances per tile (zero before the count)
     uint32_t *tile_cur;            // [tiles] fill cursor of each tile
     uint32_t *tile_last;           // [tiles] the forward's largest n_contrib per tile: zeroed here
     uint2 *ranges;                 // [tiles] [start, end) of each tile's list
@@ -59,11 +61,11 @@ struct BinBlock {
     unsigned long long warp[kBinThreads / 32];
 };
 
-// Instance j (block-local, below the block's total) of the block: its record
-// slot in the block and its global tile id.
-__device__ __forceinline__ uint32_t bin_instance(const BinBlock &s, unsigned long long j, int &slot)
+// Instance j (block-local, below the block's total) of the block's recs
+// records: its record slot in the block and its global tile id.
+__device__ __forceinline__ uint32_t bin_instance(const BinBlock &s, unsigned long long j, int recs, int &slot)
 {
-    int lo = 0, hi = kBinThreads - 1; // first record whose inclusive prefix exceeds j
+    int lo = 0, hi = recs - 1; // first record whose inclusive prefix exceeds j
     while (lo < hi) {
         const int mid = (lo + hi) >> 1;
         if (s.incl[mid] > j) hi = mid; else lo = mid + 1;
@@ -103,38 +105,45 @@ __device__ __forceinline__ unsigned long long bin_load(const BinArgs &a, const C
 }
 
 // 1. Count: each record's first instance (record order) and every tile's count.
+// Persistent blocks take chunks of kBinThreads records by ticket, as many as
+// there are records (not as many as the capacity could hold).
 __global__ void __launch_bounds__(kBinThreads) bin_count_kernel(BinArgs a, const CamTable *__restrict__ ctp)
 {
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
     __shared__ BinBlock s;
     __shared__ unsigned s_bid;
     __shared__ unsigned long long s_base;
-    if (threadIdx.x == 0) s_bid = atomicAdd((unsigned *)a.lb_count, 1u); // blocks in ticket order
-    __syncthreads();
-    const unsigned bid = s_bid;
     const unsigned long long nrec = a.ctr->n_records;
-    const unsigned long long k0 = (unsigned long long)bid * kBinThreads;
-    if (k0 >= nrec) return;
-    unsigned long long c, total;
-    const unsigned long long excl = bin_load(a, *ctp, s, k0, nrec, kBinThreads, c, total);
-    if (threadIdx.x < 32) {
-        const unsigned long long b = lookback_exclusive(a.lb_count + 1, bid, total, a.ctr, kSiteEmit);
-        if (threadIdx.x == 0) s_base = b;
-    }
-    __syncthreads();
-    const unsigned long long base = s_base;
-    const unsigned long long k = k0 + threadIdx.x;
-    if (k < nrec) a.inst_off[k] = (uint32_t)(base + excl);
-    if (k == nrec - 1) {
-        const unsigned long long end = base + excl + c;
-        a.ctr->instances_needed = end;
-        a.ctr->n_instances = end < a.max_instances ? end : a.max_instances;
-        if (end > a.max_instances) set_error(a.ctr, GS_ERR_CAPACITY, kSiteEmit);
-    }
-    for (unsigned long long j = threadIdx.x; j < total; j += kBinThreads) {
-        int slot;
-        const uint32_t t = bin_instance(s, j, slot);
-        atomicAdd(&a.tile_cnt[t], 1u);
+    if (nrec == 0 && blockIdx.x == 0 && threadIdx.x == 0) a.ctr->instances_needed = a.ctr->n_instances = 0ull;
+    for (;;) {
+        if (threadIdx.x == 0) s_bid = atomicAdd((unsigned *)a.lb_count, 1u); // chunks in ticket order
+        __syncthreads();
+        const unsigned bid = s_bid;
+        const unsigned long long k0 = (unsigned long long)bid * kBinThreads;
+        if (k0 >= nrec) return;
+        unsigned long long c, total;
+        const unsigned long long excl = bin_load(a, *ctp, s, k0, nrec, kBinThreads, c, total);
+        if (threadIdx.x == 0) lookback_publish(a.lb_count + 1, bid, total);
+        for (unsigned long long j = threadIdx.x; j < total; j += kBinThreads) {
+            int slot;
+            const uint32_t t = bin_instance(s, j, kBinThreads, slot);
+            atomicAdd(&a.tile_cnt[t], 1u);
+        }
+        if (threadIdx.x < 32) {
+            const unsigned long long b = lookback_resolve(a.lb_count + 1, bid, total, a.ctr, kSiteEmit);
+            if (threadIdx.x == 0) s_base = b;
+        }
+        __syncthreads();
+        const unsigned long long base = s_base;
+        const unsigned long long k = k0 + threadIdx.x;
+        if (k < nrec) a.inst_off[k] = (uint32_t)(base + excl);
+        if (k == nrec - 1) {
+            const unsigned long long end = base + excl + c;
+            a.ctr->instances_needed = end;
+            a.ctr->n_instances = end < a.max_instances ? end : a.max_instances;
+            if (end > a.max_instances) set_error(a.ctr, GS_ERR_CAPACITY, kSiteEmit);
+        }
+        __syncthreads(); // every thread is done with this chunk's shared values
     }
 }
 
@@ -174,46 +183,55 @@ __global__ void __launch_bounds__(256) tile_scan_kernel(BinArgs a)
         a.ranges[t0 + q] = make_uint2((uint32_t)min(off, a.max_instances), (uint32_t)min(e, a.max_instances));
         a.tile_cur[t0 + q] = (uint32_t)min(off, a.max_instances);
         a.tile_last[t0 + q] = 0u;
+        a.tile_cnt[t0 + q] = 0u; // for the next binning
         off = e;
     }
 }
 
 // 3. Scatter: every instance to the next position of its tile.  A block of
-// kBinThreads threads takes kScatterRecs records, so that twice as many
-// cursor atomics are in flight per SM as records per thread would allow.
+// kBinThreads threads takes kScatterRecs records at a time, so that twice as
+// many cursor atomics are in flight per SM as records per thread would allow;
+// blocks stride over the records there are.  The count pass's look-back words
+// are cleared for the next binning.
 __global__ void __launch_bounds__(kBinThreads) bin_scatter_kernel(BinArgs a, const CamTable *__restrict__ ctp)
 {
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
     __shared__ BinBlock s;
     const unsigned long long nrec = a.ctr->n_records;
-    const unsigned long long k0 = (unsigned long long)blockIdx.x * kScatterRecs;
-    if (k0 >= nrec) return;
-    unsigned long long c, total;
-    bin_load(a, *ctp, s, k0, nrec, kScatterRecs, c, total);
-    // four instances per round: their cursor atomics are in flight together
-    constexpr int kRound = 4;
-    for (unsigned long long j0 = threadIdx.x; j0 < total; j0 += kRound * kBinThreads) {
-        uint32_t pos[kRound], r[kRound], end[kRound], dk[kRound];
+    const unsigned long long words = (nrec + kBinThreads - 1) / kBinThreads + 1;
+    for (unsigned long long w = (unsigned long long)blockIdx.x * kBinThreads + threadIdx.x; w < words;
+         w += (unsigned long long)gridDim.x * kBinThreads)
+        a.lb_count[w] = 0ull;
+    for (unsigned long long k0 = (unsigned long long)blockIdx.x * kScatterRecs; k0 < nrec;
+         k0 += (unsigned long long)gridDim.x * kScatterRecs) {
+        unsigned long long c, total;
+        bin_load(a, *ctp, s, k0, nrec, kScatterRecs, c, total);
+        // four instances per round: their cursor atomics are in flight together
+        constexpr int kRound = 4;
+        for (unsigned long long j0 = threadIdx.x; j0 < total; j0 += kRound * kBinThreads) {
+            uint32_t pos[kRound], r[kRound], end[kRound], dk[kRound];
 #pragma unroll
-        for (int q = 0; q < kRound; q++) { // every load and atomic of the round issued first
-            const unsigned long long j = j0 + (unsigned long long)q * kBinThreads;
-            if (j >= total) break;
-            int slot;
-            const uint32_t t = bin_instance(s, j, slot);
-            r[q] = s.rec[slot];
-            pos[q] = atomicAdd(&a.tile_cur[t], 1u);
-            end[q] = a.ranges[t].y;
-            dk[q] = a.dkey[r[q]];
-        }
+            for (int q = 0; q < kRound; q++) { // every load and atomic of the round issued first
+                const unsigned long long j = j0 + (unsigned long long)q * kBinThreads;
+                if (j >= total) break;
+                int slot;
+                const uint32_t t = bin_instance(s, j, kScatterRecs, slot);
+                r[q] = s.rec[slot];
+                pos[q] = atomicAdd(&a.tile_cur[t], 1u);
+                end[q] = a.ranges[t].y;
+                dk[q] = a.dkey[r[q]];
+            }
 #pragma unroll
-        for (int q = 0; q < kRound; q++) {
-            const unsigned long long j = j0 + (unsigned long long)q * kBinThreads;
-            if (j >= total) break;
-            if (pos[q] < end[q]) { // within the capacity-clamped range
-                a.skey[pos[q]] = dk[q];
-                a.sval[pos[q]] = r[q];
+            for (int q = 0; q < kRound; q++) {
+                const unsigned long long j = j0 + (unsigned long long)q * kBinThreads;
+                if (j >= total) break;
+                if (pos[q] < end[q]) { // within the capacity-clamped range
+                    a.skey[pos[q]] = dk[q];
+                    a.sval[pos[q]] = r[q];
+                }
             }
         }
+        __syncthreads(); // every thread is done with these records' shared values
     }
 }
 
@@ -317,6 +335,10 @@ __global__ void __launch_bounds__(32 * kTileSortWarps, 8) tile_sort_kernel(BinAr
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long t = (long long)blockIdx.x * kTileSortWarps + warp;
     if (t >= a.total_tiles) return;
+    if (lane == 0 && t % (256 * kTileScanItems) == 0) { // the tile scan's look-back words, for the next binning
+        a.lb_tiles[1 + t / (256 * kTileScanItems)] = 0ull;
+        if (t == 0) a.lb_tiles[0] = 0ull;
+    }
     const uint2 rg = a.ranges[t];
     const uint32_t start = rg.x, n = rg.y - rg.x;
     if (n <= 1) return; // a single record is in place
@@ -359,28 +381,28 @@ __global__ void __launch_bounds__(32 * kTileSortWarps, 8) tile_sort_kernel(BinAr
 
 // The tile lists of the records of the last preprocess: ranges and
 // ws->tval[0] (records sorted by (tile, depth bits, record)), inst_off, the
-// instance counters.  Scratch: tile_cnt, tile_cur, the two look-back regions
-// of lb_status, tkey[0..1], tval[1].
+// instance counters.  Scratch: tile_cnt, tile_cur, bin_lb, tkey[0..1], tval[1].
+// tile_cnt and bin_lb are zero between calls: the pass after the last reader
+// clears them, so a binning needs no memset.
 cudaError_t launch_bin(gs_workspace *ws, cudaStream_t st)
 {
     const unsigned long long rcap = (unsigned long long)ws->cap.max_records;
     const int tiles = ws->cams.total_tiles;
-    const unsigned cblocks = (unsigned)((rcap + kBinThreads - 1) / kBinThreads);
+    const unsigned long long cblocks = (rcap + kBinThreads - 1) / kBinThreads;
     const unsigned sblocks = (unsigned)((tiles + 256 * kTileScanItems - 1) / (256 * kTileScanItems));
     const size_t lb_need = (size_t)cblocks + 1 + sblocks + 1;
-    if (lb_need > ws->lb_words) return cudaErrorInvalidValue; // sized at creation
-    cudaError_t e;
-    if ((e = cudaMemsetAsync(ws->lb_status, 0, lb_need * sizeof(unsigned long long), st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(ws->tile_cnt, 0, (size_t)tiles * sizeof(uint32_t), st)) != cudaSuccess) return e;
+    if (lb_need > ws->bin_lb_words) return cudaErrorInvalidValue; // sized at creation
+    // as many blocks as stay resident, striding over the records
+    const unsigned long long resident = 16ull * ws->sm_count;
     BinArgs a;
     a.tt = ws->tt; a.rect = ws->rect; a.rec_cam = ws->rec_cam; a.dkey = ws->dkey;
     a.inst_off = ws->inst_off; a.tile_cnt = ws->tile_cnt; a.tile_cur = ws->tile_cur; a.ranges = ws->ranges;
     a.tile_last = ws->tile_last;
     a.skey = ws->tkey[0]; a.sval = ws->tval[0]; a.xkey = ws->tkey[1]; a.xval = ws->tval[1];
-    a.lb_count = ws->lb_status; a.lb_tiles = ws->lb_status + cblocks + 1;
+    a.lb_count = ws->bin_lb; a.lb_tiles = ws->bin_lb + cblocks + 1;
     a.ctr = ws->ctr; a.max_instances = (unsigned long long)ws->cap.max_instances; a.total_tiles = tiles;
     kt_begin(ws, GS_KT_BIN_COUNT, st);
-    launch_pdl(bin_count_kernel, cblocks, kBinThreads, 0, st, a, ws->d_cams);
+    launch_pdl(bin_count_kernel, (unsigned)std::max(1ull, std::min(cblocks, resident)), kBinThreads, 0, st, a, ws->d_cams);
     kt_end(ws, GS_KT_BIN_COUNT, st);
     note_launch();
     kt_begin(ws, GS_KT_BIN_SORT, st);
@@ -388,8 +410,8 @@ cudaError_t launch_bin(gs_workspace *ws, cudaStream_t st)
         launch_pdl(tile_scan_kernel, sblocks, 256, 0, st, a);
         note_launch();
     }
-    launch_pdl(bin_scatter_kernel, (unsigned)((rcap + kScatterRecs - 1) / kScatterRecs), kBinThreads, 0, st, a,
-               ws->d_cams);
+    const unsigned long long scat = (rcap + kScatterRecs - 1) / kScatterRecs;
+    launch_pdl(bin_scatter_kernel, (unsigned)std::max(1ull, std::min(scat, 12ull * ws->sm_count)), kBinThreads, 0, st, a, ws->d_cams);
     note_launch();
     if (tiles > 0) {
         launch_pdl(tile_sort_kernel, (unsigned)((tiles + kTileSortWarps - 1) / kTileSortWarps), 32 * kTileSortWarps,

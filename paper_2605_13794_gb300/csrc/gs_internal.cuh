@@ -207,20 +207,23 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v)
     return v;
 }
 
-// Called by one full warp of block `bid`.  Publishes the block aggregate,
-// walks back over predecessors 32 at a time and returns the exclusive prefix
-// of this block (to every lane), then publishes the inclusive prefix.  Every
-// wait is bounded: on timeout the error word is set and the walk stops.
-__device__ __forceinline__ unsigned long long lookback_exclusive(unsigned long long *status, unsigned bid,
-                                                                 unsigned long long aggregate, DevCounters *ctr,
-                                                                 int site)
+// Look-back of block `bid` in two halves, so that a block can publish its
+// aggregate as soon as it has it and do other work before it needs its prefix:
+// lookback_publish (one thread), then lookback_resolve (one full warp), which
+// walks back over the predecessors 32 at a time, returns the exclusive prefix
+// of the block (to every lane) and publishes the inclusive one.  Every wait is
+// bounded: on timeout the error word is set and the walk stops.
+__device__ __forceinline__ void lookback_publish(unsigned long long *status, unsigned bid, unsigned long long aggregate)
+{
+    lb_store(&status[bid], (bid == 0 ? kLbInc : kLbAgg) | aggregate);
+}
+
+__device__ __forceinline__ unsigned long long lookback_resolve(unsigned long long *status, unsigned bid,
+                                                               unsigned long long aggregate, DevCounters *ctr,
+                                                               int site)
 {
     const int lane = threadIdx.x & 31;
-    if (bid == 0) {
-        if (lane == 0) lb_store(&status[0], kLbInc | aggregate);
-        return 0ull;
-    }
-    if (lane == 0) lb_store(&status[bid], kLbAgg | aggregate);
+    if (bid == 0) return 0ull;
     unsigned long long excl = 0;
     long long pred = (long long)bid - 1;
     while (true) {
@@ -252,6 +255,15 @@ __device__ __forceinline__ unsigned long long lookback_exclusive(unsigned long l
     }
     if (lane == 0) lb_store(&status[bid], kLbInc | (excl + aggregate));
     return excl;
+}
+
+// Both halves, by one full warp of block `bid`.
+__device__ __forceinline__ unsigned long long lookback_exclusive(unsigned long long *status, unsigned bid,
+                                                                 unsigned long long aggregate, DevCounters *ctr,
+                                                                 int site)
+{
+    if ((threadIdx.x & 31) == 0) lookback_publish(status, bid, aggregate);
+    return lookback_resolve(status, bid, aggregate, ctr, site);
 }
 
 // Block-wide exclusive scan of one value per thread, NW warps per block.
@@ -343,9 +355,10 @@ struct gs_workspace {
     // per Gaussian (candidates of the gate stage, in index order)
     uint32_t *cand_g;              // [N]
     unsigned long long *cand_mask; // [N] bit per camera
-    uint32_t *gate_g;              // [N] block-strided candidates of the gate's first pass
+    uint16_t *gate_cnt;            // [N / 128] candidates of each chunk of the gate
+    uint32_t *gate_g;              // [N] the gate's candidates, each chunk's at the start of its own range
     unsigned long long *gate_mask; // [N]
-    uint32_t *rec_first;           // [N] first record of each Gaussian, ~0 when none
+    uint32_t *rec_first;           // [N] dense Adam from compact rows: first record of each Gaussian, ~0 when none
     float *cgrad;                  // [R][59] compact gradient rows (fused backward + Adam)
     // per record
     uint32_t *rec_g;
@@ -359,7 +372,7 @@ struct gs_workspace {
     uint8_t *clampm;
     float *rgrad;        // [R][9] per-record summed gradients of u v A B C o r g b
     uint32_t *dkey;      // [R] FP32 bits of each record's camera depth
-    uint32_t *tile_cnt, *tile_cur; // [T] the binning's tile counts and fill cursors
+    uint32_t *tile_cnt, *tile_cur; // [T] the binning's tile counts (zero between calls) and fill cursors
     uint32_t *tile_last;           // [T] largest n_contrib of each tile's pixels (zeroed by the binning, set by the forward)
     // per instance
     uint32_t *tkey[2], *tval[2];
@@ -382,8 +395,10 @@ struct gs_workspace {
     float *loss_partial; // [2 * blocks]
     size_t loss_partial_words;
     // scan / sort scratch
-    unsigned long long *lb_status; // [max(blocks)+1] single-value look-back + ticket
+    unsigned long long *lb_status; // preprocess: look-back + ticket of the gather and the projection
     size_t lb_words;
+    unsigned long long *bin_lb;    // binning: look-back + ticket of the count and the tile scan; zero between calls
+    size_t bin_lb_words;
     uint32_t *rx_status; // radix: [4][256] histograms, then per pass [blocks * 256 + 1] look-back + ticket
     size_t rx_words;
     uint32_t *rx_hist;   // [4][256]: the first kRxHistWords words of rx_status (also a scratch of 1024 words)

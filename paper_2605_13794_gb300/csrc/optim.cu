@@ -587,7 +587,6 @@ enum LazyMode { kLazyAll = 0, kLazyCandidates = 1, kLazyGrad = 2 };
 struct LazyItems {
     const uint32_t *cand_g;    // kLazyCandidates: the catch-up list (Gaussians of the gate's candidates that are behind)
     const uint32_t *rec_g;     // kLazyGrad: Gaussian of each record (a Gaussian's records contiguous)
-    const uint32_t *rec_first; // kLazyGrad: first record of each Gaussian
     const float *cgrad;        // kLazyGrad: compact gradient rows at the first record
     const DevCounters *ctr;    // sizes of the device lists
     long long n;               // kLazyAll: Gaussians
@@ -836,7 +835,7 @@ static gs_gaussian_grads params_of(const gs_gaussians &g)
 static LazyItems lazy_items(gs_workspace *ws, long long n)
 {
     LazyItems it;
-    it.cand_g = ws->cand_g; it.rec_g = ws->rec_g; it.rec_first = ws->rec_first; it.cgrad = ws->cgrad;
+    it.cand_g = ws->cand_g; it.rec_g = ws->rec_g; it.cgrad = ws->cgrad;
     it.ctr = ws->ctr; it.n = n;
     return it;
 }
@@ -923,6 +922,16 @@ static cudaError_t launch_lazy_adam(gs_workspace *ws, cudaStream_t st, const gs_
     return launch_lazy_list<kLazyGrad>(ws, st, lazy_args(ws, param, n), (unsigned long long)ws->cap.max_records);
 }
 
+// First record of each Gaussian with records, for the dense pass's lookups.
+__global__ void __launch_bounds__(256) first_records_kernel(const uint32_t *rec_g, uint32_t *rec_first,
+                                                            const DevCounters *ctr)
+{
+    griddep_wait(); // programmatic dependent launch: the previous kernel is complete
+    const unsigned long long nrec = ctr->n_records;
+    for (unsigned long long r = (unsigned long long)blockIdx.x * 256 + threadIdx.x; r < nrec; r += gridDim.x * 256ull)
+        if (r == 0 || rec_g[r - 1] != rec_g[r]) rec_first[rec_g[r]] = (uint32_t)r;
+}
+
 cudaError_t launch_adam_sparse(gs_workspace *ws, cudaStream_t st, const gs_gaussian_grads &param,
                                const gs_gaussian_grads &m, const gs_gaussian_grads &v, long long n,
                                const float lr[5], float beta1, float beta2, float eps, int step)
@@ -934,6 +943,11 @@ cudaError_t launch_adam_sparse(gs_workspace *ws, cudaStream_t st, const gs_gauss
                                        ws->ctr);
     note_launch();
     if (ws->lazy.enabled) return launch_lazy_adam(ws, st, param, n);
+    cudaError_t e = cudaMemsetAsync(ws->rec_first, 0xff, (size_t)n * sizeof(uint32_t), st);
+    if (e != cudaSuccess) return e;
+    launch_pdl(first_records_kernel, lazy_grid(ws, (unsigned long long)ws->cap.max_records), 256, 0, st, ws->rec_g,
+               ws->rec_first, (const DevCounters *)ws->ctr);
+    note_launch();
     AdamTable t;
     t.n = 5;
     t.cgrad = ws->cgrad;

@@ -128,28 +128,6 @@ __device__ __forceinline__ bool lod_pass(const float m[3], int lod, const CamInf
     return d2 <= thr2[lod];
 }
 
-// lod_pass for a mean that may still move by up to D (deferred Adam steps):
-// passes whenever some point within D of m passes.  D = 0 is lod_pass.
-__device__ __forceinline__ bool lod_pass_margin(const float m[3], int lod, const CamInfo &cam, const RenderConsts &rc,
-                                                const float *thr2, const float *thr, float D)
-{
-    if (D == 0.f) return lod_pass(m, lod, cam, rc, thr2);
-    if (!rc.lod_enable || lod == 0) return true;
-    if (lod > rc.lod_Lmax) return false;
-    const float dx = m[0] - cam.campos[0], dy = m[1] - cam.campos[1], dz = m[2] - cam.campos[2];
-    const float lim = 1.0001f * (thr[lod] + D);
-    return dx * dx + dy * dy + dz * dz <= lim * lim;
-}
-
-// Depth row of camera_point alone (the near-plane test).
-__device__ __forceinline__ void camera_z(const float m[3], const CamInfo &cam, float &tz, float &ez)
-{
-    const float *R = cam.R;
-    tz = FADD(FADD(FADD(FMUL(R[6], m[0]), FMUL(R[7], m[1])), FMUL(R[8], m[2])), cam.t[2]);
-    const float mag = fabsf(R[6] * m[0]) + fabsf(R[7] * m[1]) + fabsf(R[8] * m[2]) + fabsf(cam.t[2]);
-    ez = 8.f * 5.9604645e-8f * mag + 1e-30f;
-}
-
 // Camera-space mean in float, for the gate only, with a bound on its distance
 // from the double-float value the projection uses: three additions and
 // the final rounding each err by at most 2^-24 of a partial sum bounded by
@@ -348,8 +326,7 @@ struct PreOut {
     uint32_t *gate_g;              // [N] block-strided candidates of the gate's first pass
     unsigned long long *gate_mask; // [N]
     const float *drift;            // [2][N] drift bounds (mean, log-scale) of deferred Adam steps, or NULL
-    uint32_t *rec_first;           // first record of each Gaussian, ~0 when it has none
-    unsigned long long *lb_status; // word 0: ticket
+    unsigned long long *lb_status; // the projection's look-back, word 0: ticket (cleared by the gate)
     DevCounters *ctr;
     long long max_records;
     const uint32_t *cull;
@@ -372,9 +349,6 @@ __device__ __forceinline__ void load_shape(const GaussPtrs &g, long long i, Gaus
     L.have_shape = true;
 }
 
-constexpr int kGateItems = 4; // Gaussians per thread of the gate kernel: 1024 per block
-static_assert((kGateItems * 8) % 32 == 0, "the gate ranks its (item, warp) counts with one warp");
-
 __device__ __forceinline__ bool cull_bit(const PreOut &o, int c, long long i)
 {
     return o.cull ? ((o.cull[c * o.cull_words + (i >> 5)] >> (i & 31)) & 1u) : false;
@@ -395,72 +369,46 @@ __device__ __forceinline__ void stage_cameras(const CamTable &ct, CamInfo *s_cam
 // plane and the conservative screen test -- everything that is cheap and
 // rejects most of a city scene -- producing an order-preserving list of
 // candidate Gaussians with a bit per camera that may still be active.
-// The Gaussians come in chunks of kGateChunk; thread t of the block that takes
-// chunk c owns Gaussians c*kGateChunk + k*256 + t.  What every test needs
-// (mean, level, mean drift) streams in: either as bulk copies of the chunk into
-// shared memory, double-buffered so that the next chunk is in flight while this
-// one is tested (persistent blocks), or, where the arrays are not 16-byte
-// aligned, as plain loads issued up front.  The log-scales (and their drift)
-// are read only for the few Gaussians past the LOD and near tests.
-constexpr int kGateChunk = 256 * kGateItems;
+// Warps work on their own, on chunks of kGateChunk consecutive Gaussians (lane
+// l owns items l, l + 32, ...).  What the first test needs (mean, level, mean
+// drift) streams in: as bulk copies of the chunk into the warp's buffer in
+// shared memory, two chunks deep, so that the next chunk is in flight while
+// this one is tested, or, where the arrays are not 16-byte aligned (and in a
+// last partial chunk), as plain loads into it.
+// Per camera the LOD test of every item costs eight instructions; the few
+// (item, camera) pairs that pass (a tenth of a city scene's) are queued, and
+// whenever 32 wait, the warp takes them through the near plane, their shape
+// (log-scales, their drift) and the screen test together, with full warps,
+// whatever camera they belong to.  Testing every camera of an item to its end
+// before the next (divergent from the first camera that one lane passes) took
+// 548 us on 4M Gaussians and 24 cameras, this 190; blocks of 1024 Gaussians
+// with block barriers took 38 us on 5M and one camera, this 31 (88 MB: 13 us).
+constexpr int kGateItems = 4;                  // items per lane
+constexpr int kGateChunk = 32 * kGateItems;    // Gaussians per chunk
+constexpr int kGateWarps = 8;                  // warps per block
+constexpr int kGateQueue = kGateChunk + 32;    // (item, camera) pairs a warp may hold
 
-struct GateShared {
-    CamInfo cams[GS_MAX_CAMERAS];
-    float thr2[kMaxLod + 1];
-    float thr[kMaxLod + 1];  // sqrt of thr2, for the drift margin
-    unsigned cnt[kGateItems][8];
-    unsigned total;
-    uint16_t surv[8][kGateChunk / 8]; // one camera: each warp's items past the LOD and near tests
-    unsigned hit[8][kGateItems];      // one camera: (warp, item) bits by lane of the candidates
-};
-
-// One chunk as the bulk copies leave it in shared memory.
-struct GateStage {
+// One chunk in shared memory.
+struct __align__(16) GateStage {
     float mean[3 * kGateChunk];
     float drift[kGateChunk];     // drift bound of the mean (deferred Adam steps)
     uint8_t lod[kGateChunk];
 };
 
-struct GateItems {
-    float mx[kGateItems], my[kGateItems], mz[kGateItems];
-    int lod[kGateItems];
-    uint32_t cw[kGateItems]; // the Cull word of camera 0 (GS_CULL_DROP)
-    float dm[kGateItems];    // drift bound of the mean, 0 when up to date
+template <bool kOneCam> struct GateWarp {
+    GateStage stage[2];
+    uint16_t queue[kGateQueue];  // item | camera << 8
+    // cameras of each item that pass every test: bits by camera, or (one camera) by item
+    uint32_t hit[kOneCam ? kGateItems : 2 * kGateChunk];
+    unsigned long long bar[2];
 };
 
-__device__ __forceinline__ void gate_load_plain(const GaussPtrs &g, const PreOut &o, const RenderConsts &rc,
-                                                long long block0, GateItems &it)
-{
-    const long long n = g.n;
-#pragma unroll
-    for (int k = 0; k < kGateItems; k++) {
-        const long long i = block0 + k * 256 + threadIdx.x;
-        const bool ok = i < n;
-        it.mx[k] = ok ? g.mean[3 * i] : 0.f;
-        it.my[k] = ok ? g.mean[3 * i + 1] : 0.f;
-        it.mz[k] = ok ? g.mean[3 * i + 2] : 0.f;
-        it.lod[k] = (ok && rc.lod_enable && g.lod) ? (int)g.lod[i] : 0;
-        it.cw[k] = (ok && rc.cull_enable == GS_CULL_DROP && o.cull) ? o.cull[i >> 5] : 0u;
-        it.dm[k] = (ok && o.drift) ? o.drift[i] : 0.f;
-    }
-}
-
-// A whole chunk (every item below n) from its staged copy.
-__device__ __forceinline__ void gate_load_staged(const GateStage &sg, const GaussPtrs &g, const PreOut &o,
-                                                 const RenderConsts &rc, long long block0, GateItems &it)
-{
-#pragma unroll
-    for (int k = 0; k < kGateItems; k++) {
-        const int j = k * 256 + threadIdx.x;
-        const long long i = block0 + j;
-        it.mx[k] = sg.mean[3 * j];
-        it.my[k] = sg.mean[3 * j + 1];
-        it.mz[k] = sg.mean[3 * j + 2];
-        it.lod[k] = (rc.lod_enable && g.lod) ? (int)sg.lod[j] : 0;
-        it.cw[k] = (rc.cull_enable == GS_CULL_DROP && o.cull) ? o.cull[i >> 5] : 0u;
-        it.dm[k] = o.drift ? sg.drift[j] : 0.f;
-    }
-}
+template <bool kOneCam> struct GateShared {
+    CamInfo cams[kOneCam ? 1 : GS_MAX_CAMERAS];
+    float thr2[kMaxLod + 1];
+    float thr[kMaxLod + 1];      // sqrt of thr2, for the drift margin
+    GateWarp<kOneCam> warp[kGateWarps];
+};
 
 // Issues the bulk copies of chunk c (a whole chunk) into sg, completing on bar.
 __device__ __forceinline__ void gate_issue(GateStage &sg, unsigned long long *bar, const GaussPtrs &g,
@@ -474,255 +422,211 @@ __device__ __forceinline__ void gate_issue(GateStage &sg, unsigned long long *ba
     if (drift) bulk_copy_g2s(sg.drift, o.drift + kGateChunk * c, 4u * kGateChunk, bar);
 }
 
-// sg: the chunk's staged copy (bulk copies), or nullptr (plain loads)
-template <bool kOneCam>
-__device__ __forceinline__ void gate_masks(const GaussPtrs &g, const PreOut &o, const CamTable &ct,
-                                           const RenderConsts &rc, GateShared &sh, long long block0,
-                                           const GateItems &it, const GateStage *sg,
-                                           unsigned long long mask[kGateItems])
+// The near plane and the screen test of the pair `code` of the chunk at
+// first, staged in sg; also the Cull column (GS_CULL_DROP).
+__device__ __forceinline__ bool gate_pair(const GaussPtrs &g, const PreOut &o, const CamInfo *cams, int tw, int th,
+                                          const RenderConsts &rc, const GateStage &sg, long long first, unsigned code)
 {
-    const int ncam = ct.n, tw = ct.tile_w, th = ct.tile_h;
-    const long long n = g.n;
-    if (kOneCam) {
-        // one camera: the LOD, Cull and near tests of every item; the few items
-        // still in (a twentieth of a city scene) are compacted per warp, in
-        // item order, and the warp's lanes take them together through their
-        // shape (log-scales, their drift) and the screen test
-        const CamInfo &cam = sh.cams[0];
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        const unsigned lt = (1u << lane) - 1u;
-        unsigned nsurv = 0;
-#pragma unroll
-        for (int k = 0; k < kGateItems; k++) {
-            const long long i = block0 + k * 256 + threadIdx.x;
-            const float m[3] = {it.mx[k], it.my[k], it.mz[k]};
-            const bool lod_ok = lod_pass_margin(m, it.lod[k], cam, rc, sh.thr2, sh.thr, it.dm[k]);
-            const bool culled = rc.cull_enable == GS_CULL_DROP && ((it.cw[k] >> (i & 31)) & 1u);
-            float tz, ez;
-            camera_z(m, cam, tz, ez);
-            const bool near_ok = tz + ez + it.dm[k] > rc.znear; // the exact near test is the projection's
-            const bool in = i < n && lod_ok && !culled && near_ok;
-            const unsigned b = __ballot_sync(0xffffffffu, in);
-            if (in) sh.surv[warp][nsurv + __popc(b & lt)] = (uint16_t)(k * 256 + threadIdx.x);
-            nsurv += __popc(b);
-        }
-        if (lane < kGateItems) sh.hit[warp][lane] = 0u;
-        __syncwarp();
-        for (unsigned q = lane; q < nsurv; q += 32) {
-            const int j = sh.surv[warp][q]; // chunk-local item: k * 256 + warp * 32 + its lane
-            const long long i = block0 + j;
-            float m[3], dm;
-            if (sg) {
-                m[0] = sg->mean[3 * j]; m[1] = sg->mean[3 * j + 1]; m[2] = sg->mean[3 * j + 2];
-                dm = o.drift ? sg->drift[j] : 0.f;
-            } else {
-                m[0] = g.mean[3 * i]; m[1] = g.mean[3 * i + 1]; m[2] = g.mean[3 * i + 2];
-                dm = o.drift ? o.drift[i] : 0.f;
-            }
-            const float dl = o.drift ? o.drift[n + i] : 0.f;
-            const float lsmax = fmaxf(g.log_scale[3 * i], fmaxf(g.log_scale[3 * i + 1], g.log_scale[3 * i + 2])) + dl;
-            float t[3], te[3];
-            camera_point(m, cam, t, te);
-            te[0] += dm; te[1] += dm; te[2] += dm;
-            const float smax = 1.0001f * __expf(lsmax);
-            if (maybe_on_screen(t, te, smax, cam, tw, th, rc)) atomicOr(&sh.hit[warp][j >> 8], 1u << (j & 31));
-        }
-        __syncwarp();
-#pragma unroll
-        for (int k = 0; k < kGateItems; k++) mask[k] = (sh.hit[warp][k] >> lane) & 1u;
-    } else {
-#pragma unroll
-        for (int k = 0; k < kGateItems; k++) {
-            mask[k] = 0;
-            const long long i = block0 + k * 256 + threadIdx.x;
-            if (i >= n) continue;
-            const float m[3] = {it.mx[k], it.my[k], it.mz[k]};
-            const float dm = it.dm[k];
-            float smax = -1.f;
-            for (int c = 0; c < ncam; c++) {
-                const CamInfo &cam = sh.cams[c];
-                if (!lod_pass_margin(m, it.lod[k], cam, rc, sh.thr2, sh.thr, dm)) continue;
-                if (rc.cull_enable == GS_CULL_DROP && (c == 0 ? ((it.cw[k] >> (i & 31)) & 1u) : cull_bit(o, c, i)))
-                    continue;
-                float t[3], te[3];
-                camera_point(m, cam, t, te);
-                te[0] += dm; te[1] += dm; te[2] += dm;
-                if (!(t[2] + te[2] > rc.znear)) continue; // the exact near test is the projection's
-                if (smax < 0.f) {
-                    const float dl = o.drift ? o.drift[n + i] : 0.f;
-                    smax = 1.0001f * __expf(fmaxf(g.log_scale[3 * i], fmaxf(g.log_scale[3 * i + 1],
-                                                                            g.log_scale[3 * i + 2])) + dl);
-                }
-                if (maybe_on_screen(t, te, smax, cam, tw, th, rc)) mask[k] |= 1ull << c;
-            }
-        }
-    }
+    const int j = code & 0xffu, c = code >> 8;
+    const long long i = first + j;
+    const CamInfo &cam = cams[c];
+    if (rc.cull_enable == GS_CULL_DROP && cull_bit(o, c, i)) return false;
+    const float m[3] = {sg.mean[3 * j], sg.mean[3 * j + 1], sg.mean[3 * j + 2]};
+    const float dm = o.drift ? sg.drift[j] : 0.f;
+    float t[3], te[3];
+    camera_point(m, cam, t, te);
+    te[0] += dm; te[1] += dm; te[2] += dm;
+    if (!(t[2] + te[2] > rc.znear)) return false; // the exact near test is the projection's
+    const float dl = o.drift ? o.drift[g.n + i] : 0.f;
+    const float lsmax = fmaxf(g.log_scale[3 * i], fmaxf(g.log_scale[3 * i + 1], g.log_scale[3 * i + 2])) + dl;
+    return maybe_on_screen(t, te, 1.0001f * __expf(lsmax), cam, tw, th, rc);
 }
 
-// Block-local order of the candidates: item (k, thread) precedes (k', thread')
-// iff k < k', or k == k' and thread < thread'.  Returns the block's count.
-__device__ __forceinline__ unsigned gate_ranks(const unsigned long long mask[kGateItems], unsigned bal[kGateItems],
-                                               GateShared &sh)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < kGateItems; k++) {
-        bal[k] = __ballot_sync(0xffffffffu, mask[k] != 0);
-        if (lane == 0) sh.cnt[k][warp] = __popc(bal[k]);
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) { // warp 0: exclusive scan of the (item, warp) counts in (k, warp) order
-        constexpr int kPer = kGateItems * 8 / 32; // consecutive counts per lane
-        unsigned c[kPer], sum = 0;
-#pragma unroll
-        for (int p = 0; p < kPer; p++) {
-            const int e = lane * kPer + p;
-            c[p] = sh.cnt[e >> 3][e & 7];
-            sum += c[p];
-        }
-        unsigned x = sum;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const unsigned y = __shfl_up_sync(0xffffffffu, x, d);
-            if (lane >= d) x += y;
-        }
-        unsigned run = x - sum;
-#pragma unroll
-        for (int p = 0; p < kPer; p++) {
-            const int e = lane * kPer + p;
-            sh.cnt[e >> 3][e & 7] = run;
-            run += c[p];
-        }
-        if (lane == 31) sh.total = x;
-    }
-    __syncthreads();
-    return sh.total;
-}
-
-// The gate runs as count, scan, gather: no block waits on another (an
-// in-order look-back chain makes the blocks of a wave, which all finish their
-// counts together, wait for one another); each chunk's candidates go first to
-// the chunk's own range, and the gather moves only candidates.
-// kBulk: persistent blocks, chunk c, c + gridDim.x, ...; the chunks copied
-// whole (all but a partial last one) arrive by bulk copies one chunk ahead.  A
-// copy that does not complete within spin_limit waits sets GS_ERR_TIMEOUT; the
-// block then waits (again bounded) for its copies in flight, records empty
-// counts for its remaining chunks and returns.
+// A warp's chunks are c, c + (warps of the grid), ...  Each chunk's candidates
+// go, in order, to the start of the chunk's own range, their number to cnt;
+// gate_gather_kernel moves them to their places in the list.  A copy that
+// does not complete within spin_limit waits sets GS_ERR_TIMEOUT; the warp then
+// waits (again bounded) for its copies in flight, records empty counts for its
+// remaining chunks and returns.  The look-back words of the kernels that
+// follow are cleared on the way.
 template <bool kOneCam, bool kBulk>
-__global__ void __launch_bounds__(256, kOneCam ? 4 : 3) gate_count_kernel(GaussPtrs g, PreOut o,
-                                                                         const CamTable *__restrict__ ctp,
-                                                                         RenderConsts rc, unsigned long long *counts,
-                                                                         unsigned long long spin_limit)
+__global__ void __launch_bounds__(32 * kGateWarps, 4) gate_count_kernel(GaussPtrs g, PreOut o,
+                                                                       const CamTable *__restrict__ ctp,
+                                                                       RenderConsts rc, uint16_t *cnt,
+                                                                       unsigned long long *lb, long long lb_words,
+                                                                       unsigned long long spin_limit)
 {
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
-    __shared__ GateShared sh;
-    __shared__ __align__(16) GateStage stage[kBulk ? 2 : 1];
-    __shared__ __align__(8) unsigned long long bar[2];
-    __shared__ int s_fail;
+    extern __shared__ __align__(16) unsigned char gate_smem[];
+    GateShared<kOneCam> &sh = *reinterpret_cast<GateShared<kOneCam> *>(gate_smem);
+    const CamTable &ct = *ctp;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    GateWarp<kOneCam> &w = sh.warp[warp];
+    const unsigned lt = (1u << lane) - 1u;
     const long long nchunks = (g.n + kGateChunk - 1) / kGateChunk;
     const long long nwhole = kBulk ? g.n / kGateChunk : 0; // chunks that come by bulk copy
+    const long long stride = (long long)gridDim.x * kGateWarps;
+    const long long c_first = (long long)blockIdx.x * kGateWarps + warp;
+    if (kBulk && lane == 0) {
+        mbar_init(&w.bar[0], 1);
+        mbar_init(&w.bar[1], 1);
+        mbar_init_fence();
+        if (c_first < nwhole) gate_issue(w.stage[0], &w.bar[0], g, o, rc, c_first);
+    }
+    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < lb_words; k += stride * 32) lb[k] = 0ull;
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int l = 0; l <= kMaxLod; l++) {
             sh.thr2[l] = rc.lod_thr2[l];
             sh.thr[l] = sqrtf(rc.lod_thr2[l]);
         }
-        s_fail = 0;
-        if (kBulk) {
-            mbar_init(&bar[0], 1);
-            mbar_init(&bar[1], 1);
-            mbar_init_fence();
-            if ((long long)blockIdx.x < nwhole) gate_issue(stage[0], &bar[0], g, o, rc, blockIdx.x);
-        }
     }
-    stage_cameras(*ctp, sh.cams); // ends with a block barrier
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned lt = (1u << lane) - 1u;
+    stage_cameras(ct, sh.cams); // ends with a block barrier, the only one
+    const int ncam = kOneCam ? 1 : ct.n, tw = ct.tile_w, th = ct.tile_h;
     int k = 0;
-    for (long long c = blockIdx.x; c < nchunks; c += gridDim.x, k++) {
-        const long long block0 = c * kGateChunk;
-        GateItems it;
+    for (long long c = c_first; c < nchunks; c += stride, k++) {
+        const long long first = c * kGateChunk;
+        const int here = (int)min((long long)kGateChunk, g.n - first);
+        GateStage &sg = w.stage[k & 1];
         if (kBulk && c < nwhole) {
-            const long long cn = c + gridDim.x;
+            const long long cn = c + stride;
             // the next chunk's copy, into the buffer the previous chunk used
-            if (threadIdx.x == 0 && cn < nwhole) gate_issue(stage[(k + 1) & 1], &bar[(k + 1) & 1], g, o, rc, cn);
-            if (!mbar_wait(&bar[k & 1], (unsigned)(k >> 1) & 1u, spin_limit)) {
-                set_error(o.ctr, GS_ERR_TIMEOUT, kSitePreprocess);
-                s_fail = 1;
-            }
-            __syncthreads();
-            if (s_fail) {
-                if (threadIdx.x == 0) { // the copies still in flight land before the block's memory is released
-                    mbar_wait(&bar[k & 1], (unsigned)(k >> 1) & 1u, spin_limit);
-                    if (cn < nwhole) mbar_wait(&bar[(k + 1) & 1], (unsigned)((k + 1) >> 1) & 1u, spin_limit);
+            if (lane == 0 && cn < nwhole) gate_issue(w.stage[(k + 1) & 1], &w.bar[(k + 1) & 1], g, o, rc, cn);
+            const bool ok = mbar_wait(&w.bar[k & 1], (unsigned)(k >> 1) & 1u, spin_limit);
+            if (__any_sync(0xffffffffu, !ok)) {
+                if (lane == 0) { // the copies still in flight land before the block's memory is released
+                    set_error(o.ctr, GS_ERR_TIMEOUT, kSitePreprocess);
+                    mbar_wait(&w.bar[k & 1], (unsigned)(k >> 1) & 1u, spin_limit);
+                    if (cn < nwhole) mbar_wait(&w.bar[(k + 1) & 1], (unsigned)((k + 1) >> 1) & 1u, spin_limit);
                 }
-                for (long long r = c + threadIdx.x * (long long)gridDim.x; r < nchunks; r += 256ll * gridDim.x)
-                    counts[r] = 0;
+                for (long long r = c + lane * stride; r < nchunks; r += 32 * stride) cnt[r] = 0;
                 return;
             }
-            gate_load_staged(stage[k & 1], g, o, rc, block0, it);
         } else {
-            gate_load_plain(g, o, rc, block0, it);
-        }
-        unsigned long long mask[kGateItems];
-        unsigned bal[kGateItems];
-        gate_masks<kOneCam>(g, o, *ctp, rc, sh, block0, it, (kBulk && c < nwhole) ? &stage[k & 1] : nullptr, mask);
-        const unsigned total = gate_ranks(mask, bal, sh);
-        if (threadIdx.x == 0) counts[c] = total;
-        // the chunk's candidates, in order, at the start of its own range
-#pragma unroll
-        for (int q = 0; q < kGateItems; q++) {
-            if (mask[q]) {
-                const long long pos = block0 + sh.cnt[q][warp] + __popc(bal[q] & lt);
-                o.gate_g[pos] = (uint32_t)(block0 + q * 256 + threadIdx.x);
-                o.gate_mask[pos] = mask[q];
+            for (int e = lane; e < 3 * here; e += 32) sg.mean[e] = g.mean[3 * first + e];
+            for (int e = lane; e < here; e += 32) {
+                if (rc.lod_enable && g.lod) sg.lod[e] = g.lod[first + e];
+                if (o.drift) sg.drift[e] = o.drift[first + e];
             }
         }
-        __syncthreads(); // the staged chunk and the ranks are free for the next chunk
+        if (kOneCam) {
+            if (lane < kGateItems) w.hit[lane] = 0u;
+        } else {
+#pragma unroll
+            for (int q = 0; q < 2 * kGateItems; q++) w.hit[q * 32 + lane] = 0u;
+        }
+        __syncwarp();
+        // the items' means and the squared-distance limits of their LOD test (Eq. 1-2): infinite
+        // where it always passes, negative where it cannot; widened past the rounding of the fused
+        // evaluation below, and by the distance a mean may still move (deferred Adam steps) -- the
+        // projection decides exactly
+        float mx[kGateItems], my[kGateItems], mz[kGateItems], lim[kGateItems];
+#pragma unroll
+        for (int q = 0; q < kGateItems; q++) {
+            const int j = 32 * q + lane;
+            mx[q] = my[q] = mz[q] = 0.f;
+            lim[q] = -1.f;
+            if (j >= here) continue;
+            mx[q] = sg.mean[3 * j]; my[q] = sg.mean[3 * j + 1]; mz[q] = sg.mean[3 * j + 2];
+            const int lod = (rc.lod_enable && g.lod) ? (int)sg.lod[j] : 0;
+            if (!rc.lod_enable || lod == 0) lim[q] = INFINITY;
+            else if (lod <= rc.lod_Lmax) {
+                const float dm = o.drift ? sg.drift[j] : 0.f, d = 1.0001f * (sh.thr[lod] + dm);
+                lim[q] = dm == 0.f ? 1.000001f * sh.thr2[lod] : d * d;
+            }
+        }
+        unsigned n = 0; // pairs in the queue
+        for (int cam = 0; cam < ncam; cam++) {
+            const float cx = sh.cams[cam].campos[0], cy = sh.cams[cam].campos[1], cz = sh.cams[cam].campos[2];
+            unsigned add = 0;
+#pragma unroll
+            for (int q = 0; q < kGateItems; q++) {
+                const float dx = mx[q] - cx, dy = my[q] - cy, dz = mz[q] - cz;
+                const bool in = lim[q] == INFINITY || fmaf(dx, dx, fmaf(dy, dy, dz * dz)) <= lim[q];
+                const unsigned b = __ballot_sync(0xffffffffu, in);
+                if (b) {
+                    if (in) w.queue[n + add + __popc(b & lt)] = (uint16_t)((32 * q + lane) | (cam << 8));
+                    add += __popc(b);
+                }
+            }
+            n += add;
+            // full warps of pairs, from the queue's end; what is left of them after the last camera
+            while (n >= 32 || (cam == ncam - 1 && n > 0)) {
+                __syncwarp();
+                const unsigned take = min(n, 32u);
+                n -= take;
+                if (lane < take) {
+                    const unsigned code = w.queue[n + lane];
+                    if (gate_pair(g, o, sh.cams, tw, th, rc, sg, first, code)) {
+                        const int j = code & 0xffu, cc = code >> 8;
+                        if (kOneCam) atomicOr(&w.hit[j >> 5], 1u << (j & 31));
+                        else atomicOr(&w.hit[2 * j + (cc >> 5)], 1u << (cc & 31));
+                    }
+                }
+                __syncwarp();
+            }
+        }
+        __syncwarp();
+        unsigned run = 0;
+#pragma unroll
+        for (int q = 0; q < kGateItems; q++) {
+            const int j = 32 * q + lane;
+            const unsigned long long mask = kOneCam ? (unsigned long long)((w.hit[q] >> lane) & 1u)
+                                                    : ((unsigned long long)w.hit[kOneCam ? 0 : 2 * j + 1] << 32) |
+                                                          w.hit[kOneCam ? 0 : 2 * j];
+            const unsigned b = __ballot_sync(0xffffffffu, mask != 0ull);
+            if (mask != 0ull) {
+                const long long pos = first + run + __popc(b & lt);
+                o.gate_g[pos] = (uint32_t)(first + j);
+                if (!kOneCam) o.gate_mask[pos] = mask;
+            }
+            run += __popc(b);
+        }
+        if (lane == 0) cnt[c] = (uint16_t)run;
+        __syncwarp(); // the buffer and the masks are free for the next chunk
     }
 }
 
-// Exclusive scan of the block counts in place (one block); the total is the
-// candidate count.
-__global__ void __launch_bounds__(1024) gate_scan_kernel(unsigned long long *counts, long long nblocks,
-                                                         DevCounters *ctr)
+// The ordered list from the chunks' candidates.  A block (in ticket order)
+// takes kGatherChunks chunks: it scans their counts, finds its offset by
+// decoupled look-back (every block publishes after the same little work) and
+// moves its candidates, the loads of four of a thread's in flight together.
+constexpr int kGatherChunks = 64;
+static_assert(kGatherChunks <= 256, "one chunk per thread of the scan");
+template <bool kOneCam>
+__global__ void __launch_bounds__(256) gate_gather_kernel(PreOut o, const uint16_t *cnt, long long nchunks,
+                                                          unsigned long long *lb /* ticket at word 0 */)
 {
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
-    __shared__ unsigned long long s[1024];
-    const long long per = (nblocks + 1023) / 1024;
-    const long long b0 = (long long)threadIdx.x * per;
-    unsigned long long acc = 0;
-    for (long long b = b0; b < b0 + per && b < nblocks; b++) acc += counts[b];
-    s[threadIdx.x] = acc;
+    __shared__ unsigned s_incl[256];
+    __shared__ unsigned s_warp[8];
+    __shared__ unsigned s_bid;
+    __shared__ unsigned long long s_base;
+    if (threadIdx.x == 0) s_bid = atomicAdd((unsigned *)lb, 1u);
     __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        const unsigned long long v = threadIdx.x >= off ? s[threadIdx.x - off] : 0ull;
-        __syncthreads();
-        s[threadIdx.x] += v;
-        __syncthreads();
+    const unsigned bid = s_bid;
+    const long long c0 = (long long)bid * kGatherChunks, c = c0 + threadIdx.x;
+    const unsigned mine = threadIdx.x < kGatherChunks && c < nchunks ? cnt[c] : 0u;
+    unsigned total;
+    const unsigned excl = block_exclusive_scan_256<unsigned>(mine, s_warp, total);
+    s_incl[threadIdx.x] = excl + mine;
+    if (threadIdx.x < 32) {
+        const unsigned long long b = lookback_exclusive(lb + 1, bid, total, o.ctr, kSitePreprocess);
+        if (threadIdx.x == 0) {
+            s_base = b;
+            if (c0 + kGatherChunks >= nchunks) o.ctr->n_candidates = b + total;
+        }
     }
-    unsigned long long run = s[threadIdx.x] - acc; // exclusive prefix of this chunk
-    for (long long b = b0; b < b0 + per && b < nblocks; b++) {
-        const unsigned long long c = counts[b];
-        counts[b] = run;
-        run += c;
-    }
-    if (threadIdx.x == 1023) ctr->n_candidates = s[1023];
-}
-
-// Moves each block's candidates from its own range to their place in the
-// ordered list (offsets from gate_scan_kernel).
-__global__ void __launch_bounds__(256) gate_gather_kernel(PreOut o, const unsigned long long *offsets,
-                                                          long long nblocks, const DevCounters *ctr)
-{
-    griddep_wait(); // programmatic dependent launch: the previous kernel is complete
-    const long long b = blockIdx.x;
-    const unsigned long long off = offsets[b];
-    const unsigned long long end = b + 1 < nblocks ? offsets[b + 1] : ctr->n_candidates;
-    const long long src = b * 256 * kGateItems;
-    for (unsigned long long t = threadIdx.x; off + t < end; t += 256) {
-        o.cand_g[off + t] = o.gate_g[src + t];
-        o.cand_mask[off + t] = o.gate_mask[src + t];
+    __syncthreads();
+    const unsigned long long base = s_base;
+#pragma unroll 4
+    for (unsigned t = threadIdx.x; t < total; t += 256) {
+        int lo = 0; // the first chunk whose inclusive count exceeds t
+#pragma unroll
+        for (int step = kGatherChunks / 2; step > 0; step >>= 1) lo += s_incl[lo + step - 1] <= t ? step : 0;
+        const long long src = (c0 + lo) * kGateChunk + (t - (lo ? s_incl[lo - 1] : 0u));
+        o.cand_g[base + t] = o.gate_g[src];
+        if (!kOneCam) o.cand_mask[base + t] = o.gate_mask[src];
     }
 }
 
@@ -832,7 +736,7 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(GaussPtrs g, PreO
     Proj p_one; // one camera: the projection of the active record
     if (j < ncand) {
         i = o.cand_g[j];
-        const unsigned long long cm = o.cand_mask[j];
+        const unsigned long long cm = kOneCam ? 1ull : o.cand_mask[j];
         L.m[0] = g.mean[3 * i]; L.m[1] = g.mean[3 * i + 1]; L.m[2] = g.mean[3 * i + 2];
         load_shape(g, i, L);
         const float ol = g.opacity_logit[i];
@@ -860,16 +764,19 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(GaussPtrs g, PreO
             const int c = __ffsll((long long)mm) - 1;
             if (cull_bit(o, c, i)) marked |= 1ull << c;
         }
+    unsigned long long total;
+    const unsigned long long excl = block_exclusive_scan<kNW, unsigned long long>(cnt, s_warp, total);
+    const int tvis = __syncthreads_count((act & ~marked) != 0);
+    // the chunk's count is published before the colours are read, so that no
+    // later chunk's look-back waits for them
+    if (threadIdx.x == 0) lookback_publish(o.lb_status + 1, bid, total);
     RecOut one;
     if (kOneCam && act) one = make_record(g, i, L, op, s_cams[0], p_one, rc, marked & 1ull);
-    unsigned long long total, tvis;
-    const unsigned long long excl = block_exclusive_scan<kNW, unsigned long long>(cnt, s_warp, total);
-    block_exclusive_scan<kNW, unsigned long long>((unsigned long long)((act & ~marked) != 0), s_warp, tvis);
     if (threadIdx.x < 32) {
-        const unsigned long long b = lookback_exclusive(o.lb_status + 1, bid, total, o.ctr, kSitePreprocess);
+        const unsigned long long b = lookback_resolve(o.lb_status + 1, bid, total, o.ctr, kSitePreprocess);
         if (threadIdx.x == 0) {
             s_base = b;
-            if (tvis) atomicAdd(&o.ctr->n_visible, tvis); // the visible set of Eq. 5
+            if (tvis) atomicAdd(&o.ctr->n_visible, (unsigned long long)tvis); // the visible set of Eq. 5
         }
     }
     __syncthreads();
@@ -880,7 +787,6 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(GaussPtrs g, PreO
         o.ctr->n_records = end < (unsigned long long)o.max_records ? end : o.max_records;
     }
     if (act) {
-        if (base < (unsigned long long)o.max_records) o.rec_first[i] = (uint32_t)base;
         if (kOneCam) {
             if (base >= (unsigned long long)o.max_records) set_error(o.ctr, GS_ERR_CAPACITY, kSitePreprocess);
             else store_record(o, base, i, 0, one);
@@ -907,54 +813,60 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(GaussPtrs g, PreO
 
 static bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
+template <bool kOneCam>
+static cudaError_t launch_gate(gs_workspace *ws, cudaStream_t st, const GaussPtrs &gp, const PreOut &o, bool bulk,
+                               unsigned long long *lb, long long lb_words)
+{
+    const size_t smem = sizeof(GateShared<kOneCam>);
+    const auto kernel = bulk ? gate_count_kernel<kOneCam, true> : gate_count_kernel<kOneCam, false>;
+    if (smem > 48u << 10) { // above the default limit
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    // persistent warps: four blocks per SM stay resident at the register budget
+    const long long chunks = (gp.n + kGateChunk - 1) / kGateChunk, blocks = (chunks + kGateWarps - 1) / kGateWarps;
+    const unsigned grid = (unsigned)std::min<long long>(blocks, 4ll * ws->sm_count);
+    const unsigned long long spins = kSpinLimit;
+    kt_begin(ws, GS_KT_GATE, st);
+    launch_pdl(kernel, grid, 32 * kGateWarps, smem, st, gp, o, ws->d_cams, ws->rc, ws->gate_cnt, lb, lb_words, spins);
+    kt_end(ws, GS_KT_GATE, st);
+    note_launch();
+    launch_pdl(gate_gather_kernel<kOneCam>, (unsigned)((chunks + kGatherChunks - 1) / kGatherChunks), 256, 0, st, o,
+               ws->gate_cnt, chunks, lb);
+    note_launch();
+    return cudaGetLastError();
+}
+
 cudaError_t launch_preprocess(gs_workspace *ws, cudaStream_t st, const uint32_t *cull)
 {
     const long long n = ws->g.n;
-    const unsigned gblocks = (unsigned)((n + kGateChunk - 1) / kGateChunk); // chunks
     const unsigned pchunks = (unsigned)((n + kProjThreads - 1) / kProjThreads); // projection chunks (at most)
     cudaError_t e;
-    // counters, then the look-back state of each stage (ticket in word 0)
     if ((e = cudaMemsetAsync(ws->ctr, 0, sizeof(DevCounters), st)) != cudaSuccess) return e;
     if (n == 0) return cudaSuccess;
     GaussPtrs gp{ws->g.mean, ws->g.log_scale, ws->g.quat, ws->g.opacity_logit, ws->g.sh, ws->g.lod, n};
+    // look-back state (ticket in word 0 of each): the gather's, then the
+    // projection's; the gate clears both
+    const long long gather_words = (n + kGateChunk * kGatherChunks - 1) / (kGateChunk * kGatherChunks) + 1;
+    const long long lb_words = gather_words + pchunks + 1;
+    if ((size_t)lb_words > ws->lb_words) return cudaErrorInvalidValue; // sized at creation
     PreOut o;
     o.rec_g = ws->rec_g; o.tt = ws->tt; o.dkey = ws->dkey;
     o.rec_cam = ws->rec_cam; o.rd0 = ws->rd0; o.rd1 = ws->rd1; o.rd2 = ws->rd2; o.rect = ws->rect;
-    o.clampm = ws->clampm; o.cand_g = ws->cand_g; o.cand_mask = ws->cand_mask; o.rec_first = ws->rec_first;
+    o.clampm = ws->clampm; o.cand_g = ws->cand_g; o.cand_mask = ws->cand_mask;
     o.gate_g = ws->gate_g; o.gate_mask = ws->gate_mask;
     o.drift = ws->lazy.enabled ? ws->lazy.drift : nullptr;
-    o.lb_status = ws->lb_status;
+    o.lb_status = ws->lb_status + gather_words;
     o.ctr = ws->ctr; o.max_records = ws->cap.max_records;
     o.cull = ws->rc.cull_enable ? cull : nullptr;
     o.cull_words = (n + 31) / 32;
-    if ((e = cudaMemsetAsync(ws->rec_first, 0xff, (size_t)n * sizeof(uint32_t), st)) != cudaSuccess) return e;
-    // gate: per-block counts (in lb_status) and candidates (block-strided), the
-    // scan of the counts, the gather into one ordered list
-    kt_begin(ws, GS_KT_GATE, st);
     // the camera count of the upload (a captured graph replays uploads of the
     // same count); bulk copies where every streamed array is 16-byte aligned
     const bool one = ws->cams.n == 1;
-    const bool bulk = n >= kGateChunk && aligned16(gp.mean) && (!gp.lod || aligned16(gp.lod)) &&
-                      (!o.drift || aligned16(o.drift));
-    const unsigned per_sm = one ? 4u : 3u;
-    const unsigned ggrid = bulk ? std::min<unsigned>(gblocks, per_sm * (unsigned)ws->sm_count) : gblocks;
-    const unsigned long long spins = kSpinLimit;
-    if (one && bulk)
-        launch_pdl(gate_count_kernel<true, true>, ggrid, 256, 0, st, gp, o, ws->d_cams, ws->rc, ws->lb_status, spins);
-    else if (one)
-        launch_pdl(gate_count_kernel<true, false>, ggrid, 256, 0, st, gp, o, ws->d_cams, ws->rc, ws->lb_status, spins);
-    else if (bulk)
-        launch_pdl(gate_count_kernel<false, true>, ggrid, 256, 0, st, gp, o, ws->d_cams, ws->rc, ws->lb_status, spins);
-    else
-        launch_pdl(gate_count_kernel<false, false>, ggrid, 256, 0, st, gp, o, ws->d_cams, ws->rc, ws->lb_status, spins);
-    kt_end(ws, GS_KT_GATE, st);
-    note_launch();
-    launch_pdl(gate_scan_kernel, 1, 1024, 0, st, ws->lb_status, (long long)gblocks, ws->ctr);
-    note_launch();
-    launch_pdl(gate_gather_kernel, gblocks, 256, 0, st, o, ws->lb_status, (long long)gblocks, ws->ctr);
-    note_launch();
-    if ((e = cudaMemsetAsync(ws->lb_status, 0, (pchunks + 1) * sizeof(unsigned long long), st)) != cudaSuccess)
-        return e;
+    const bool bulk = aligned16(gp.mean) && (!gp.lod || aligned16(gp.lod)) && (!o.drift || aligned16(o.drift));
+    e = one ? launch_gate<true>(ws, st, gp, o, bulk, ws->lb_status, lb_words)
+            : launch_gate<false>(ws, st, gp, o, bulk, ws->lb_status, lb_words);
+    if (e != cudaSuccess) return e;
     // deferred Adam steps: bring the candidates up to date before projecting them
     if (ws->lazy.enabled && (e = launch_lazy_catchup(ws, st, ws->g)) != cudaSuccess) return e;
     // projection: persistent blocks, about as many as stay resident (five per
