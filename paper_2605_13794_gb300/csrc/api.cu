@@ -46,8 +46,8 @@ struct Layout {
 };
 
 struct Offsets {
-    size_t cand_g, cand_mask, gate_cnt, gate_g, gate_mask, rec_first, cgrad, rec_g, rec_cam, rd0, rd1, rd2, rect, tt, inst_off, clampm, rgrad, dkey, tile_cnt, tile_cur, tile_last;
-    size_t tkey0, tkey1, tval0, tval1, slots, imp_slots, ranges, n_contrib, T_final, imp_w, imp_a, sel_cum, sel_bsum;
+    size_t cand_g, cand_mask, gate_cnt, gate_g, gate_mask, rec_first, cgrad, rec_g, rec_cam, rd0, rd1, rd2, rect, tt, inst_off, chunk_rec, clampm, rgrad, dkey, tile_cnt, tile_last;
+    size_t pairs, inst_rank, sval, slots, imp_slots, ranges, n_contrib, T_final, imp_w, imp_a, sel_cum, sel_bsum;
     size_t selk0, selk1, selv0, selv1, loss_maps, loss_partial, lb_status, bin_lb, rx_status, red_partial,
         ctr, d_cams, d_adam_step, d_adam_coef;
     size_t mkey0, mkey1, mval0, mval1, mcum, mbsum, mrx_status, mlb, mhist, mctr;
@@ -77,18 +77,17 @@ Offsets plan(const gs_capacity &c)
     o.rect = L.take<uint2>(R);
     o.tt = L.take<uint32_t>(R);
     o.inst_off = L.take<uint32_t>(R);
+    o.chunk_rec = L.take<uint32_t>(I / gs::kBinChunk + 2);
     o.clampm = L.take<uint8_t>(R);
     o.rgrad = L.take<float>(fwd_only ? 0 : R * gs::kSlotFloats);
     o.dkey = L.take<uint32_t>(R);
-    o.tkey0 = L.take<uint32_t>(I);
-    o.tkey1 = L.take<uint32_t>(I);
-    o.tval0 = L.take<uint32_t>(I);
-    o.tval1 = L.take<uint32_t>(I);
+    o.pairs = L.take<uint2>(I);
+    o.inst_rank = L.take<uint32_t>(I);
+    o.sval = L.take<uint32_t>(I);
     o.slots = L.take<float>(fwd_only ? 0 : I * gs::kSlotFloats);
     o.imp_slots = L.take<float2>(I); // importance (w, a) per instance
     o.ranges = L.take<uint2>(T);
     o.tile_cnt = L.take<uint32_t>(T);
-    o.tile_cur = L.take<uint32_t>(T);
     o.tile_last = L.take<uint32_t>(T);
     o.n_contrib = L.take<uint32_t>(P);
     o.T_final = L.take<float>(P);
@@ -103,12 +102,11 @@ Offsets plan(const gs_capacity &c)
     o.loss_maps = L.take<float>(fwd_only ? 0 : P * 3 * 3); // per pixel and channel: F0, F1, F2 (planar)
     o.loss_partial_words = fwd_only ? 0 : 2 * 3 * (P / 1024 + 65536);
     o.loss_partial = L.take<float>(o.loss_partial_words);
-    // look-back words of the preprocess: one per 128 candidates of the
+    // look-back words of the preprocess: two per 128 candidates of the
     // projection, one per 8192 Gaussians of the gather, and their tickets
-    o.lb_words = N / 128 + N / 8192 + 8;
+    o.lb_words = 2 * (N / 128) + N / 8192 + 10;
     o.lb_status = L.take<unsigned long long>(o.lb_words);
-    // ... of the binning: 128 records of its count pass, 1024 tiles of its scan
-    o.bin_lb_words = R / 128 + T / 1024 + 8;
+    o.bin_lb_words = T / 1024 + 4; // ... of the binning: 1024 tiles of its scan
     o.bin_lb = L.take<unsigned long long>(o.bin_lb_words);
     const size_t items = (R > I ? R : I);
     // the histograms, then the look-back state of up to four passes, for the
@@ -279,14 +277,15 @@ int gs_workspace_create(const gs_capacity *cap, gs_workspace **out)
     ws->rect = (uint2 *)(b + o.rect);
     ws->tt = (uint32_t *)(b + o.tt);
     ws->inst_off = (uint32_t *)(b + o.inst_off);
+    ws->chunk_rec = (uint32_t *)(b + o.chunk_rec);
     ws->clampm = (uint8_t *)(b + o.clampm);
     ws->rgrad = (float *)(b + o.rgrad);
     ws->dkey = (uint32_t *)(b + o.dkey);
     ws->tile_cnt = (uint32_t *)(b + o.tile_cnt);
-    ws->tile_cur = (uint32_t *)(b + o.tile_cur);
     ws->tile_last = (uint32_t *)(b + o.tile_last);
-    ws->tkey[0] = (uint32_t *)(b + o.tkey0); ws->tkey[1] = (uint32_t *)(b + o.tkey1);
-    ws->tval[0] = (uint32_t *)(b + o.tval0); ws->tval[1] = (uint32_t *)(b + o.tval1);
+    ws->pairs = (uint2 *)(b + o.pairs);
+    ws->inst_rank = (uint32_t *)(b + o.inst_rank);
+    ws->sval = (uint32_t *)(b + o.sval);
     ws->slots = (float *)(b + o.slots);
     ws->imp_slots = (float2 *)(b + o.imp_slots);
     ws->ranges = (uint2 *)(b + o.ranges);
@@ -558,7 +557,6 @@ int gs_bin_sort(gs_workspace *ws, gs_stream stream)
     // tile counts, ranges, scatter and the per-tile depth sort (the final
     // order: camera, tile, depth bits, record)
     CK(gs::launch_bin(ws, st), "gs_bin_sort");
-    ws->tile_buf = 0;
     ws->have_binning = 1;
     ws->imp_ready = 0;
     return GS_OK;
@@ -943,7 +941,7 @@ int gs_workspace_buffer(gs_workspace *ws, int32_t which, void **ptr, int64_t *co
     case GS_BUF_REC_XY_CONIC: *ptr = ws->rd0; *count = c.max_records; break;
     case GS_BUF_REC_C_OPAC_RG: *ptr = ws->rd1; *count = c.max_records; break;
     case GS_BUF_REC_B_LO: *ptr = ws->rd2; *count = c.max_records; break;
-    case GS_BUF_SORTED_VALUES: *ptr = ws->tval[ws->tile_buf]; *count = c.max_instances; break;
+    case GS_BUF_SORTED_VALUES: *ptr = ws->sval; *count = c.max_instances; break;
     case GS_BUF_TILE_RANGES: *ptr = ws->ranges; *count = c.max_tiles; break;
     case GS_BUF_N_CONTRIB: *ptr = ws->n_contrib; *count = c.max_pixels; break;
     default: return fail(GS_ERR_INVALID_ARG, "gs_workspace_buffer: unknown buffer %d", which);

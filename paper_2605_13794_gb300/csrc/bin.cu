@@ -3,20 +3,26 @@
 // inside each tile.
 //
 // Order of the work:
-//   1. count: records in record order ((Gaussian, camera) order), blocks of
-//      kBinThreads; a block scans its records' tile counts and finds its
-//      global offset by a decoupled look-back, so each record's first
-//      instance (inst_off, the base of its gradient slots) follows record
-//      order; every instance adds one to its tile's count;
+//   1. count: every instance adds one to its tile's count and keeps the count
+//      it found, its rank in the tile (in whatever order they came).  The
+//      projection numbers the instances in record order ((Gaussian, camera)
+//      order, inst_off, the base of the gradient slots); blocks take equal
+//      chunks of them, so a record of thousands of tiles is spread over many;
 //   2. tile scan: exclusive scan of the tile counts (decoupled look-back over
-//      blocks of tiles) gives each tile's range and a fill cursor;
-//   3. scatter: every instance takes the next position of its tile (an
-//      atomic on the cursor) and writes its record and depth key there;
-//   4. per-tile sort: one warp per tile sorts the tile's (depth bits,
-//      record) pairs -- unique keys, so the order is the same in any
-//      scatter order -- in registers (a bitonic network over shuffles, up
-//      to kTileSortMax entries) or, for a longer list, in chunks merged
-//      through a scratch copy in global memory.
+//      blocks of tiles) gives each tile's range;
+//   3. scatter: every instance writes its (depth key, record) pair at its
+//      tile's start plus its rank;
+//   4. per-tile sort of the (depth bits, record) pairs -- unique keys, so the
+//      order is the same in any scatter order -- in registers (bitonic
+//      networks over shuffles): up to kWarpSort entries in one warp, up to
+//      kBlockSort in the four warps of a block, which then rank their runs
+//      against each other, longer lists in sorted chunks merged through a
+//      scratch copy in global memory.
+// Bound by the latency of atomics and scattered stores.  Dealing out records
+// (32 to a warp or block) left whole SMs waiting for the blocks that held
+// records of hundreds of tiles: the count and scatter of the 1.14M instances
+// of the 5M city at 1080p took 17 + 24 us and take 13 + 11 in equal chunks of
+// instances, the 11.2M of 24 mixed views 78 + 233 us and 95 + 147.
 // The final order of a tile's list is (depth bits, record): depth ties go to
 // the lower record, i.e. the lower Gaussian index.  Counts stay on the
 // device; nothing here synchronises with the host.
@@ -26,130 +32,128 @@
 
 namespace gs {
 
-constexpr int kBinThreads = 128;       // threads (and records) per block of the count pass
-constexpr int kScatterRecs = 32;       // records per block of the scatter pass (kBinThreads threads)
+constexpr int kBinThreads = 128;       // threads per block of the count and scatter passes
+constexpr int kBinItems = kBinChunk / kBinThreads; // instances per thread
 constexpr int kTileScanItems = 4;      // tiles per thread of the tile scan (1024 per block)
-constexpr int kTileSortMax = 512;      // entries a warp sorts in registers (16 per lane)
-constexpr int kTileSortWarps = 4;      // tiles per block of the per-tile sort
+constexpr int kSortWarps = 4;          // warps (and tiles) per block of the per-tile sort
+constexpr int kWarpSort = 128;         // entries one warp sorts alone (4 per lane)
+constexpr int kBlockSort = 2048;       // entries a block sorts in shared memory (16 per lane)
 
 struct BinArgs {
     const uint32_t *tt;
     const uint2 *rect;
     const uint16_t *rec_cam;
     const uint32_t *dkey;          // FP32 bits of each record's camera depth
-    uint32_t *inst_off;            // first instance of each record (record order)
+    const uint32_t *inst_off;      // first instance of each record (record order)
+    const uint32_t *chunk_rec;     // record of each chunk's first instance
+    uint32_t *rank;                // [instances] rank of each instance among those of its tile
     uint32_t *tile_cnt;            // [tiles] instances per tile (zero before the count)
-    uint32_t *tile_cur;            // [tiles] fill cursor of each tile
     uint32_t *tile_last;           // [tiles] the forward's largest n_contrib per tile: zeroed here
     uint2 *ranges;                 // [tiles] [start, end) of each tile's list
-    uint32_t *skey, *sval;         // [instances] scattered depth keys and records; sval ends sorted
-    uint32_t *xkey, *xval;         // [instances] scratch of the merges of long lists
-    unsigned long long *lb_count;  // look-back of the count pass (ticket at word 0)
+    uint2 *pairs;                  // [instances] scattered (depth key, record) pairs
+    uint32_t *sval;                // [instances] the sorted records
+    uint2 *scratch;                // [instances] scratch of the merges of long lists
     unsigned long long *lb_tiles;  // look-back of the tile scan (ticket at word 0)
     DevCounters *ctr;
     unsigned long long max_instances;
     int total_tiles;
 };
 
-// The records of one block of the count or scatter pass in shared memory:
-// inclusive prefix of their tile counts, rectangle and camera tile layout.
-struct BinBlock {
-    unsigned long long incl[kBinThreads];
-    uint32_t rec[kBinThreads];
-    uint2 rect[kBinThreads];
-    int tile_base[kBinThreads], tiles_x[kBinThreads];
-    unsigned long long warp[kBinThreads / 32];
+// The records of one chunk of kBinChunk consecutive instances, in shared memory.
+struct BinRecs {
+    uint32_t off[kBinChunk + 1];   // first instance
+    uint2 rect[kBinChunk + 1];
+    int tile_base[kBinChunk + 1], tiles_x[kBinChunk + 1];
 };
 
-// Instance j (block-local, below the block's total) of the block's recs
-// records: its record slot in the block and its global tile id.
-__device__ __forceinline__ uint32_t bin_instance(const BinBlock &s, unsigned long long j, int recs, int &slot)
+// Instances of the tile lists: those of the records there are, at most the
+// capacity (more is an error, which the count pass reports).  Past the record
+// capacity (an error already) only the kept records' count.
+__device__ __forceinline__ unsigned long long bin_instances(const BinArgs &a, unsigned long long nrec,
+                                                            unsigned long long &needed)
 {
-    int lo = 0, hi = recs - 1; // first record whose inclusive prefix exceeds j
+    needed = a.ctr->inst_total;
+    if (a.ctr->records_needed > nrec) needed = nrec ? (unsigned long long)a.inst_off[nrec - 1] + a.tt[nrec - 1] : 0ull;
+    return needed < a.max_instances ? needed : a.max_instances;
+}
+
+// Loads the records of chunk b (ninst instances in all); returns the first.
+// (Whatever a projection that gave up left behind, records stay below nrec.)
+__device__ __forceinline__ uint32_t bin_load(const BinArgs &a, const CamTable &ct, BinRecs &s, unsigned long long b,
+                                             unsigned long long ninst, uint32_t nrec, uint32_t &count)
+{
+    const uint32_t r0 = min(a.chunk_rec[b], nrec - 1u);
+    const uint32_t r1 = (b + 1) * kBinChunk < ninst ? max(r0, min(a.chunk_rec[b + 1], nrec - 1u)) : nrec - 1u;
+    count = min(r1 - r0 + 1u, (uint32_t)kBinChunk + 1u);
+    for (uint32_t i = threadIdx.x; i < count; i += kBinThreads) {
+        const uint32_t r = r0 + i;
+        const int cam = a.rec_cam[r];
+        s.off[i] = a.inst_off[r];
+        s.rect[i] = a.rect[r];
+        s.tile_base[i] = ct.c[cam].tile_base;
+        s.tiles_x[i] = ct.c[cam].tiles_x;
+    }
+    __syncthreads();
+    return r0;
+}
+
+// Instance j: its record (as its slot among the chunk's) and its global tile id.
+__device__ __forceinline__ uint32_t bin_instance(const BinRecs &s, uint32_t count, uint32_t j, uint32_t &slot)
+{
+    uint32_t lo = 0, hi = count - 1; // the last record whose first instance is at most j
     while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (s.incl[mid] > j) hi = mid; else lo = mid + 1;
+        const uint32_t mid = (lo + hi + 1) >> 1;
+        if (s.off[mid] <= j) lo = mid; else hi = mid - 1;
     }
     slot = lo;
-    const unsigned long long first = lo ? s.incl[lo - 1] : 0ull;
-    const uint32_t local = (uint32_t)(j - first);
+    const uint32_t local = j - s.off[lo];
     int x0, y0, x1, y1;
     unpack_rect(s.rect[lo], x0, y0, x1, y1);
     const uint32_t w = (uint32_t)(x1 - x0);
-    const int tx = x0 + (int)(local % w), ty = y0 + (int)(local / w);
-    return (uint32_t)(s.tile_base[lo] + ty * s.tiles_x[lo] + tx);
+    // local / w: below 2^20 the rounded quotient of local + 1/2 cannot reach the
+    // next integer (its error, 2^-22 of at most 2^20 / w, is below 1 / (2 w))
+    const uint32_t q = local < (1u << 20) ? (uint32_t)__fdividef((float)local + 0.5f, (float)w) : local / w;
+    return (uint32_t)(s.tile_base[lo] + (y0 + (int)q) * s.tiles_x[lo] + x0 + (int)(local - q * w));
 }
 
-// Loads the block's records k0 .. k0 + recs - 1 (those below nrec; recs <=
-// kBinThreads, one per thread) and scans their tile counts; returns this
-// thread's exclusive prefix and the block's total.
-__device__ __forceinline__ unsigned long long bin_load(const BinArgs &a, const CamTable &ct, BinBlock &s,
-                                                       unsigned long long k0, unsigned long long nrec, int recs,
-                                                       unsigned long long &c, unsigned long long &total)
-{
-    const unsigned long long k = k0 + threadIdx.x;
-    c = 0;
-    if ((int)threadIdx.x < recs && k < nrec) {
-        const uint32_t r = (uint32_t)k;
-        c = a.tt[r];
-        const int cam = a.rec_cam[r];
-        s.rect[threadIdx.x] = a.rect[r];
-        s.tile_base[threadIdx.x] = ct.c[cam].tile_base;
-        s.tiles_x[threadIdx.x] = ct.c[cam].tiles_x;
-    }
-    s.rec[threadIdx.x] = (uint32_t)k;
-    const unsigned long long excl = block_exclusive_scan<kBinThreads / 32, unsigned long long>(c, s.warp, total);
-    s.incl[threadIdx.x] = excl + c;
-    __syncthreads();
-    return excl;
-}
-
-// 1. Count: each record's first instance (record order) and every tile's count.
-// Persistent blocks take chunks of kBinThreads records by ticket, as many as
-// there are records (not as many as the capacity could hold).
+// 1. Count: every tile's count and every instance's rank in its tile.  Blocks
+// stride over the chunks there are (not as many as the capacity could hold).
 __global__ void __launch_bounds__(kBinThreads) bin_count_kernel(BinArgs a, const CamTable *__restrict__ ctp)
 {
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
-    __shared__ BinBlock s;
-    __shared__ unsigned s_bid;
-    __shared__ unsigned long long s_base;
+    __shared__ BinRecs s;
     const unsigned long long nrec = a.ctr->n_records;
-    if (nrec == 0 && blockIdx.x == 0 && threadIdx.x == 0) a.ctr->instances_needed = a.ctr->n_instances = 0ull;
-    for (;;) {
-        if (threadIdx.x == 0) s_bid = atomicAdd((unsigned *)a.lb_count, 1u); // chunks in ticket order
-        __syncthreads();
-        const unsigned bid = s_bid;
-        const unsigned long long k0 = (unsigned long long)bid * kBinThreads;
-        if (k0 >= nrec) return;
-        unsigned long long c, total;
-        const unsigned long long excl = bin_load(a, *ctp, s, k0, nrec, kBinThreads, c, total);
-        if (threadIdx.x == 0) lookback_publish(a.lb_count + 1, bid, total);
-        for (unsigned long long j = threadIdx.x; j < total; j += kBinThreads) {
-            int slot;
-            const uint32_t t = bin_instance(s, j, kBinThreads, slot);
-            atomicAdd(&a.tile_cnt[t], 1u);
+    unsigned long long needed;
+    const unsigned long long ninst = bin_instances(a, nrec, needed);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.ctr->instances_needed = needed;
+        a.ctr->n_instances = ninst;
+        if (needed > a.max_instances) set_error(a.ctr, GS_ERR_CAPACITY, kSiteEmit);
+    }
+    for (unsigned long long b = blockIdx.x; b * kBinChunk < ninst; b += gridDim.x) {
+        uint32_t count;
+        bin_load(a, *ctp, s, b, ninst, (uint32_t)nrec, count);
+        uint32_t rank[kBinItems];
+#pragma unroll
+        for (int q = 0; q < kBinItems; q++) { // the atomics in flight together
+            const unsigned long long j = b * kBinChunk + q * kBinThreads + threadIdx.x;
+            if (j >= ninst) continue;
+            uint32_t slot;
+            const uint32_t t = bin_instance(s, count, (uint32_t)j, slot);
+            rank[q] = t < (uint32_t)a.total_tiles ? atomicAdd(&a.tile_cnt[t], 1u) : 0u;
         }
-        if (threadIdx.x < 32) {
-            const unsigned long long b = lookback_resolve(a.lb_count + 1, bid, total, a.ctr, kSiteEmit);
-            if (threadIdx.x == 0) s_base = b;
+#pragma unroll
+        for (int q = 0; q < kBinItems; q++) {
+            const unsigned long long j = b * kBinChunk + q * kBinThreads + threadIdx.x;
+            if (j < ninst) a.rank[j] = rank[q];
         }
-        __syncthreads();
-        const unsigned long long base = s_base;
-        const unsigned long long k = k0 + threadIdx.x;
-        if (k < nrec) a.inst_off[k] = (uint32_t)(base + excl);
-        if (k == nrec - 1) {
-            const unsigned long long end = base + excl + c;
-            a.ctr->instances_needed = end;
-            a.ctr->n_instances = end < a.max_instances ? end : a.max_instances;
-            if (end > a.max_instances) set_error(a.ctr, GS_ERR_CAPACITY, kSiteEmit);
-        }
-        __syncthreads(); // every thread is done with this chunk's shared values
+        __syncthreads(); // every thread is done with the chunk's records
     }
 }
 
 // 2. Tile scan: exclusive scan of the tile counts; ranges clamped to the
-// instance capacity (an overflow is already an error), cursors at the start,
-// the forward's per-tile maxima of n_contrib cleared.
+// instance capacity (an overflow is already an error); the tile counts and the
+// forward's per-tile maxima of n_contrib cleared.
 __global__ void __launch_bounds__(256) tile_scan_kernel(BinArgs a)
 {
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
@@ -181,57 +185,40 @@ __global__ void __launch_bounds__(256) tile_scan_kernel(BinArgs a)
         if (t0 + q >= a.total_tiles) break;
         const unsigned long long e = off + cnt[q];
         a.ranges[t0 + q] = make_uint2((uint32_t)min(off, a.max_instances), (uint32_t)min(e, a.max_instances));
-        a.tile_cur[t0 + q] = (uint32_t)min(off, a.max_instances);
         a.tile_last[t0 + q] = 0u;
         a.tile_cnt[t0 + q] = 0u; // for the next binning
         off = e;
     }
 }
 
-// 3. Scatter: every instance to the next position of its tile.  A block of
-// kBinThreads threads takes kScatterRecs records at a time, so that twice as
-// many cursor atomics are in flight per SM as records per thread would allow;
-// blocks stride over the records there are.  The count pass's look-back words
-// are cleared for the next binning.
+// 3. Scatter: every instance's pair to its place, one store of eight bytes.
 __global__ void __launch_bounds__(kBinThreads) bin_scatter_kernel(BinArgs a, const CamTable *__restrict__ ctp)
 {
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
-    __shared__ BinBlock s;
+    __shared__ BinRecs s;
     const unsigned long long nrec = a.ctr->n_records;
-    const unsigned long long words = (nrec + kBinThreads - 1) / kBinThreads + 1;
-    for (unsigned long long w = (unsigned long long)blockIdx.x * kBinThreads + threadIdx.x; w < words;
-         w += (unsigned long long)gridDim.x * kBinThreads)
-        a.lb_count[w] = 0ull;
-    for (unsigned long long k0 = (unsigned long long)blockIdx.x * kScatterRecs; k0 < nrec;
-         k0 += (unsigned long long)gridDim.x * kScatterRecs) {
-        unsigned long long c, total;
-        bin_load(a, *ctp, s, k0, nrec, kScatterRecs, c, total);
-        // four instances per round: their cursor atomics are in flight together
-        constexpr int kRound = 4;
-        for (unsigned long long j0 = threadIdx.x; j0 < total; j0 += kRound * kBinThreads) {
-            uint32_t pos[kRound], r[kRound], end[kRound], dk[kRound];
+    unsigned long long needed;
+    const unsigned long long ninst = bin_instances(a, nrec, needed);
+    for (unsigned long long b = blockIdx.x; b * kBinChunk < ninst; b += gridDim.x) {
+        uint32_t rank[kBinItems];
 #pragma unroll
-            for (int q = 0; q < kRound; q++) { // every load and atomic of the round issued first
-                const unsigned long long j = j0 + (unsigned long long)q * kBinThreads;
-                if (j >= total) break;
-                int slot;
-                const uint32_t t = bin_instance(s, j, kScatterRecs, slot);
-                r[q] = s.rec[slot];
-                pos[q] = atomicAdd(&a.tile_cur[t], 1u);
-                end[q] = a.ranges[t].y;
-                dk[q] = a.dkey[r[q]];
-            }
-#pragma unroll
-            for (int q = 0; q < kRound; q++) {
-                const unsigned long long j = j0 + (unsigned long long)q * kBinThreads;
-                if (j >= total) break;
-                if (pos[q] < end[q]) { // within the capacity-clamped range
-                    a.skey[pos[q]] = dk[q];
-                    a.sval[pos[q]] = r[q];
-                }
-            }
+        for (int q = 0; q < kBinItems; q++) {
+            const unsigned long long j = b * kBinChunk + q * kBinThreads + threadIdx.x;
+            rank[q] = j < ninst ? a.rank[j] : 0u;
         }
-        __syncthreads(); // every thread is done with these records' shared values
+        uint32_t count;
+        const uint32_t r0 = bin_load(a, *ctp, s, b, ninst, (uint32_t)nrec, count);
+#pragma unroll
+        for (int q = 0; q < kBinItems; q++) {
+            const unsigned long long j = b * kBinChunk + q * kBinThreads + threadIdx.x;
+            if (j >= ninst) continue;
+            uint32_t slot;
+            const uint32_t t = bin_instance(s, count, (uint32_t)j, slot);
+            if (t >= (uint32_t)a.total_tiles) continue;
+            const unsigned long long pos = (unsigned long long)a.ranges[t].x + rank[q];
+            if (pos < a.max_instances) a.pairs[pos] = make_uint2(a.dkey[r0 + slot], r0 + slot);
+        }
+        __syncthreads(); // every thread is done with the chunk's records
     }
 }
 
@@ -275,134 +262,181 @@ template <int E> __device__ __forceinline__ void warp_sort_regs(unsigned long lo
     }
 }
 
-__device__ __forceinline__ unsigned long long key_at(const uint32_t *kk, const uint32_t *vv, uint32_t i)
-{
-    return ((unsigned long long)kk[i] << 32) | vv[i];
-}
+__device__ __forceinline__ unsigned long long key_of(uint2 p) { return ((unsigned long long)p.x << 32) | p.y; }
 
 // Number of the first d outputs of the merge of X (nx) and Y (ny) that come
 // from X (merge path; keys unique).
-__device__ __forceinline__ uint32_t merge_split(const uint32_t *xk, const uint32_t *xv, uint32_t nx,
-                                                const uint32_t *yk, const uint32_t *yv, uint32_t ny, uint32_t d)
+__device__ __forceinline__ uint32_t merge_split(const uint2 *x, uint32_t nx, const uint2 *y, uint32_t ny, uint32_t d)
 {
     uint32_t lo = d > ny ? d - ny : 0u, hi = d < nx ? d : nx;
     while (lo < hi) {
         const uint32_t mid = (lo + hi) >> 1;
-        if (key_at(xk, xv, mid) < key_at(yk, yv, d - 1 - mid)) lo = mid + 1;
+        if (key_of(x[mid]) < key_of(y[d - 1 - mid])) lo = mid + 1;
         else hi = mid;
     }
     return lo;
 }
 
-// Sorts the n <= 32 * E keys (depth bits, record) at position `at` of (kk,
-// vv) -- padded with the largest key -- and writes the records (rv) or the
-// keys (rk, rv) back in order.
-template <int E>
-__device__ __forceinline__ void sort_run(const uint32_t *kk, const uint32_t *vv, uint32_t n, uint32_t *rk, uint32_t *rv)
+// The n <= 32 * E keys at p in the warp's registers, padded with the largest
+// key (in any order: consecutive lanes read consecutive keys).
+template <int E> __device__ __forceinline__ void load_keys(const uint2 *p, uint32_t n, unsigned long long (&x)[E])
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int e = 0; e < E; e++) x[e] = (uint32_t)(e * 32 + lane) < n ? key_of(p[e * 32 + lane]) : ~0ull;
+}
+
+// One warp sorts the n <= 32 * E keys at p and writes the records in order.
+template <int E> __device__ __forceinline__ void warp_sort(const uint2 *p, uint32_t n, uint32_t *out)
 {
     const int lane = threadIdx.x & 31;
     unsigned long long x[E];
-#pragma unroll
-    for (int e = 0; e < E; e++) {
-        const uint32_t g = (uint32_t)(lane * E + e);
-        x[e] = g < n ? key_at(kk, vv, g) : ~0ull;
-    }
+    load_keys<E>(p, n, x);
     warp_sort_regs<E>(x);
 #pragma unroll
-    for (int e = 0; e < E; e++) {
-        const uint32_t g = (uint32_t)(lane * E + e);
-        if (g < n) {
-            if (rk) rk[g] = (uint32_t)(x[e] >> 32);
-            rv[g] = (uint32_t)x[e];
-        }
-    }
+    for (int e = 0; e < E; e++)
+        if ((uint32_t)(lane * E + e) < n) out[lane * E + e] = (uint32_t)x[e];
 }
 
-__device__ __forceinline__ void sort_short(const uint32_t *kk, const uint32_t *vv, uint32_t n, uint32_t *rk, uint32_t *rv)
+// The block sorts the n <= 32 * E * kSortWarps keys at p: each warp a run of a
+// quarter of them, in registers, into shared memory; then every key's place is
+// its place in its run plus the keys below it in each other run (a binary
+// search; keys unique).  Writes the records to out, or the keys to outk.
+template <int E>
+__device__ __forceinline__ void block_sort(const uint2 *p, uint32_t n, unsigned long long (*s)[kBlockSort / kSortWarps],
+                                           uint32_t *out, uint2 *outk)
 {
-    if (n <= 32) sort_run<1>(kk, vv, n, rk, rv);
-    else if (n <= 64) sort_run<2>(kk, vv, n, rk, rv);
-    else if (n <= 128) sort_run<4>(kk, vv, n, rk, rv);
-    else if (n <= 256) sort_run<8>(kk, vv, n, rk, rv);
-    else sort_run<16>(kk, vv, n, rk, rv);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t run = (n + kSortWarps - 1) / kSortWarps;
+    const uint32_t first = min(warp * run, n), len = min(run, n - first);
+    {
+        unsigned long long x[E];
+        load_keys<E>(p + first, len, x);
+        warp_sort_regs<E>(x);
+#pragma unroll
+        for (int e = 0; e < E; e++) s[warp][lane * E + e] = x[e];
+    }
+    __syncthreads();
+    for (uint32_t i = lane; i < len; i += 32) {
+        const unsigned long long key = s[warp][i];
+        uint32_t place = i;
+#pragma unroll
+        for (int o = 1; o < kSortWarps; o++) {
+            const int r = (warp + o) % kSortWarps;
+            uint32_t lo = 0; // keys of run r below this one (the padding is above every key)
+#pragma unroll
+            for (uint32_t step = 16 * E; step > 0; step >>= 1) lo += s[r][lo + step - 1] < key ? step : 0;
+            lo += s[r][lo] < key ? 1u : 0u;
+            place += lo;
+        }
+        if (outk) outk[place] = make_uint2((uint32_t)(key >> 32), (uint32_t)key);
+        else out[place] = (uint32_t)key;
+    }
+    __syncthreads(); // the runs are read
 }
 
-// 4. Per-tile sort of the scattered (depth bits, record) pairs; the sorted
-// records end in sval.  One warp per tile, keys in registers.
-__global__ void __launch_bounds__(32 * kTileSortWarps, 8) tile_sort_kernel(BinArgs a)
+__device__ __forceinline__ void block_sort_any(const uint2 *p, uint32_t n,
+                                               unsigned long long (*s)[kBlockSort / kSortWarps], uint32_t *out,
+                                               uint2 *outk)
+{
+    constexpr uint32_t kRun = 32 * kSortWarps;
+    if (n <= 2 * kRun) block_sort<2>(p, n, s, out, outk);
+    else if (n <= 4 * kRun) block_sort<4>(p, n, s, out, outk);
+    else if (n <= 8 * kRun) block_sort<8>(p, n, s, out, outk);
+    else block_sort<16>(p, n, s, out, outk);
+}
+
+// 4. Per-tile sort of the scattered pairs; the sorted records end in sval.  A
+// block has kSortWarps tiles: each warp sorts its own if it is short, then the
+// whole block the longer ones, one after the other, so that a view of few
+// tiles with long lists does not wait for one warp's chain of stages.
+__global__ void __launch_bounds__(32 * kSortWarps, 8) tile_sort_kernel(BinArgs a)
 {
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
+    __shared__ unsigned long long s_run[kSortWarps][kBlockSort / kSortWarps];
+    __shared__ uint2 s_rg[kSortWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long t = (long long)blockIdx.x * kTileSortWarps + warp;
-    if (t >= a.total_tiles) return;
-    if (lane == 0 && t % (256 * kTileScanItems) == 0) { // the tile scan's look-back words, for the next binning
-        a.lb_tiles[1 + t / (256 * kTileScanItems)] = 0ull;
-        if (t == 0) a.lb_tiles[0] = 0ull;
-    }
-    const uint2 rg = a.ranges[t];
-    const uint32_t start = rg.x, n = rg.y - rg.x;
-    if (n <= 1) return; // a single record is in place
-    if (n <= (uint32_t)kTileSortMax) {
-        sort_short(a.skey + start, a.sval + start, n, nullptr, a.sval + start);
-        return;
-    }
-    // a long list: sorted chunks of kTileSortMax into the scratch, then
-    // pairwise merges of runs, the warp's lanes on equal shares of each merge
-    for (uint32_t c0 = 0; c0 < n; c0 += kTileSortMax)
-        sort_short(a.skey + start + c0, a.sval + start + c0, min((uint32_t)kTileSortMax, n - c0), a.xkey + start + c0,
-                   a.xval + start + c0);
-    const uint32_t *srck = a.xkey + start, *srcv = a.xval + start;
-    uint32_t *dstk = a.skey + start, *dstv = a.sval + start;
-    for (uint32_t width = kTileSortMax; width < n; width <<= 1) {
-        __syncwarp(); // the previous level's writes, before this level reads them
-        for (uint32_t p = 0; p < n; p += 2 * width) {
-            const uint32_t nx = min(width, n - p), ny = p + width < n ? min(width, n - p - width) : 0u;
-            const uint32_t *xk = srck + p, *xv = srcv + p, *yk = srck + p + nx, *yv = srcv + p + nx;
-            const uint32_t L = nx + ny, d0 = (uint32_t)(((unsigned long long)L * lane) / 32),
-                           d1 = (uint32_t)(((unsigned long long)L * (lane + 1)) / 32);
-            uint32_t i = merge_split(xk, xv, nx, yk, yv, ny, d0), j = d0 - i;
-            for (uint32_t d = d0; d < d1; d++) {
-                const bool take_x = j >= ny || (i < nx && key_at(xk, xv, i) < key_at(yk, yv, j));
-                const unsigned long long v = take_x ? key_at(xk, xv, i) : key_at(yk, yv, j);
-                if (take_x) i++;
-                else j++;
-                dstk[p + d] = (uint32_t)(v >> 32);
-                dstv[p + d] = (uint32_t)v;
-            }
+    const long long t = (long long)blockIdx.x * kSortWarps + warp;
+    uint2 rg = make_uint2(0u, 0u);
+    if (t < a.total_tiles) {
+        rg = a.ranges[t];
+        if (lane == 0 && t % (256 * kTileScanItems) == 0) { // the tile scan's look-back words, for the next binning
+            a.lb_tiles[1 + t / (256 * kTileScanItems)] = 0ull;
+            if (t == 0) a.lb_tiles[0] = 0ull;
         }
-        const uint32_t *tk = srck, *tv = srcv;
-        srck = dstk; srcv = dstv;
-        dstk = const_cast<uint32_t *>(tk); dstv = const_cast<uint32_t *>(tv);
     }
-    __syncwarp();
-    if (srcv != a.sval + start) // the last level wrote the scratch: the records back into sval
-        for (uint32_t i = lane; i < n; i += 32) a.sval[start + i] = srcv[i];
+    const uint32_t mine = rg.y - rg.x;
+    if (lane == 0) s_rg[warp] = rg;
+    if (mine > 0 && mine <= (uint32_t)kWarpSort) {
+        const uint2 *p = a.pairs + rg.x;
+        uint32_t *out = a.sval + rg.x;
+        if (mine <= 32) warp_sort<1>(p, mine, out);
+        else if (mine <= 64) warp_sort<2>(p, mine, out);
+        else warp_sort<4>(p, mine, out);
+    }
+    if (!__syncthreads_or(mine > (uint32_t)kWarpSort)) return;
+    for (int w = 0; w < kSortWarps; w++) {
+        const uint32_t start = s_rg[w].x, n = s_rg[w].y - start;
+        if (n <= (uint32_t)kWarpSort) continue; // the same for the whole block
+        uint2 *pairs = a.pairs + start, *scratch = a.scratch + start;
+        if (n <= (uint32_t)kBlockSort) {
+            block_sort_any(pairs, n, s_run, a.sval + start, nullptr);
+            continue;
+        }
+        // a longer list: sorted chunks of kBlockSort into the scratch, then
+        // pairwise merges of runs, the threads on equal shares of each merge
+        for (uint32_t c0 = 0; c0 < n; c0 += kBlockSort)
+            block_sort_any(pairs + c0, min((uint32_t)kBlockSort, n - c0), s_run, nullptr, scratch + c0);
+        const uint2 *src = scratch;
+        uint2 *dst = pairs;
+        constexpr uint32_t kThreads = 32 * kSortWarps;
+        for (uint32_t width = kBlockSort; width < n; width <<= 1) {
+            __syncthreads(); // the previous level's writes, before this level reads them
+            for (uint32_t p = 0; p < n; p += 2 * width) {
+                const uint32_t nx = min(width, n - p), ny = p + width < n ? min(width, n - p - width) : 0u;
+                const uint2 *x = src + p, *y = src + p + nx;
+                const uint32_t L = nx + ny, d0 = (uint32_t)(((unsigned long long)L * threadIdx.x) / kThreads),
+                               d1 = (uint32_t)(((unsigned long long)L * (threadIdx.x + 1)) / kThreads);
+                uint32_t i = merge_split(x, nx, y, ny, d0), j = d0 - i;
+                for (uint32_t d = d0; d < d1; d++) {
+                    const bool take_x = j >= ny || (i < nx && key_of(x[i]) < key_of(y[j]));
+                    dst[p + d] = take_x ? x[i] : y[j];
+                    if (take_x) i++;
+                    else j++;
+                }
+            }
+            uint2 *was = const_cast<uint2 *>(src);
+            src = dst;
+            dst = was;
+        }
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < n; i += kThreads) a.sval[start + i] = src[i].y;
+    }
 }
 
 // The tile lists of the records of the last preprocess: ranges and
-// ws->tval[0] (records sorted by (tile, depth bits, record)), inst_off, the
-// instance counters.  Scratch: tile_cnt, tile_cur, bin_lb, tkey[0..1], tval[1].
+// ws->sval (records sorted by (tile, depth bits, record)), the
+// instance counters.  Scratch: tile_cnt, bin_lb, pairs, inst_rank, and the
+// importance slots (for merges; they are written only after the binning).
 // tile_cnt and bin_lb are zero between calls: the pass after the last reader
 // clears them, so a binning needs no memset.
 cudaError_t launch_bin(gs_workspace *ws, cudaStream_t st)
 {
-    const unsigned long long rcap = (unsigned long long)ws->cap.max_records;
     const int tiles = ws->cams.total_tiles;
-    const unsigned long long cblocks = (rcap + kBinThreads - 1) / kBinThreads;
     const unsigned sblocks = (unsigned)((tiles + 256 * kTileScanItems - 1) / (256 * kTileScanItems));
-    const size_t lb_need = (size_t)cblocks + 1 + sblocks + 1;
-    if (lb_need > ws->bin_lb_words) return cudaErrorInvalidValue; // sized at creation
-    // as many blocks as stay resident, striding over the records
-    const unsigned long long resident = 16ull * ws->sm_count;
+    if ((size_t)sblocks + 1 > ws->bin_lb_words) return cudaErrorInvalidValue; // sized at creation
     BinArgs a;
     a.tt = ws->tt; a.rect = ws->rect; a.rec_cam = ws->rec_cam; a.dkey = ws->dkey;
-    a.inst_off = ws->inst_off; a.tile_cnt = ws->tile_cnt; a.tile_cur = ws->tile_cur; a.ranges = ws->ranges;
+    a.inst_off = ws->inst_off; a.chunk_rec = ws->chunk_rec; a.rank = ws->inst_rank; a.tile_cnt = ws->tile_cnt; a.ranges = ws->ranges;
     a.tile_last = ws->tile_last;
-    a.skey = ws->tkey[0]; a.sval = ws->tval[0]; a.xkey = ws->tkey[1]; a.xval = ws->tval[1];
-    a.lb_count = ws->bin_lb; a.lb_tiles = ws->bin_lb + cblocks + 1;
+    a.pairs = ws->pairs; a.sval = ws->sval; a.scratch = reinterpret_cast<uint2 *>(ws->imp_slots);
+    a.lb_tiles = ws->bin_lb;
     a.ctr = ws->ctr; a.max_instances = (unsigned long long)ws->cap.max_instances; a.total_tiles = tiles;
+    // as many blocks as stay resident, striding over the chunks
+    const unsigned long long chunks = (a.max_instances + kBinChunk - 1) / kBinChunk;
+    const unsigned rblocks = (unsigned)std::max(1ull, std::min(chunks, 16ull * ws->sm_count));
     kt_begin(ws, GS_KT_BIN_COUNT, st);
-    launch_pdl(bin_count_kernel, (unsigned)std::max(1ull, std::min(cblocks, resident)), kBinThreads, 0, st, a, ws->d_cams);
+    launch_pdl(bin_count_kernel, rblocks, kBinThreads, 0, st, a, ws->d_cams);
     kt_end(ws, GS_KT_BIN_COUNT, st);
     note_launch();
     kt_begin(ws, GS_KT_BIN_SORT, st);
@@ -410,12 +444,10 @@ cudaError_t launch_bin(gs_workspace *ws, cudaStream_t st)
         launch_pdl(tile_scan_kernel, sblocks, 256, 0, st, a);
         note_launch();
     }
-    const unsigned long long scat = (rcap + kScatterRecs - 1) / kScatterRecs;
-    launch_pdl(bin_scatter_kernel, (unsigned)std::max(1ull, std::min(scat, 12ull * ws->sm_count)), kBinThreads, 0, st, a, ws->d_cams);
+    launch_pdl(bin_scatter_kernel, rblocks, kBinThreads, 0, st, a, ws->d_cams);
     note_launch();
     if (tiles > 0) {
-        launch_pdl(tile_sort_kernel, (unsigned)((tiles + kTileSortWarps - 1) / kTileSortWarps), 32 * kTileSortWarps,
-                   0, st, a);
+        launch_pdl(tile_sort_kernel, (unsigned)((tiles + kSortWarps - 1) / kSortWarps), 32 * kSortWarps, 0, st, a);
         note_launch();
     }
     kt_end(ws, GS_KT_BIN_SORT, st);

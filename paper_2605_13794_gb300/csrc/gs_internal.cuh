@@ -60,6 +60,7 @@ constexpr size_t kRxHistWords = 4 * 256;  // radix histograms: 256 buckets for e
 constexpr int kSortThreads = 256;
 constexpr int kSortItems = 16;          // keys per thread in a radix pass (default)
 constexpr int kSortTile = kSortThreads * kSortItems;
+constexpr int kBinChunk = 256;          // instances per chunk of the binning's passes
 constexpr int kScanTile = 4096;         // items per block of the selection's prefix sums
 // per (record, tile) gradient slot, as the compositing adjoint writes it: the
 // dG-weighted moments sum dG e, sum dG dy, sum dG dx^2, sum dG dx dy, sum dG dy^2
@@ -100,6 +101,7 @@ struct DevCounters {
     unsigned long long n_visible;
     unsigned long long records_needed;
     unsigned long long instances_needed;
+    unsigned long long inst_total;     // instances of the records (the projection's count)
     unsigned long long n_candidates;   // Gaussians passing the gate stage of preprocess
     unsigned long long n_catchup;      // candidates behind the current Adam step (deferred steps to replay)
     int error;
@@ -368,17 +370,21 @@ struct gs_workspace {
     float4 *rd2;         // b, u_lo, v_lo (mean = u + u_lo), 0
     uint2 *rect;
     uint32_t *tt;
-    uint32_t *inst_off;
+    uint32_t *inst_off;  // first instance of each record
+    uint32_t *chunk_rec; // [I / kBinChunk + 1] record of each kBinChunk-th instance
     uint8_t *clampm;
     float *rgrad;        // [R][9] per-record summed gradients of u v A B C o r g b
     uint32_t *dkey;      // [R] FP32 bits of each record's camera depth
-    uint32_t *tile_cnt, *tile_cur; // [T] the binning's tile counts (zero between calls) and fill cursors
+    uint32_t *tile_cnt;            // [T] the binning's tile counts (zero between calls)
     uint32_t *tile_last;           // [T] largest n_contrib of each tile's pixels (zeroed by the binning, set by the forward)
     // per instance
-    uint32_t *tkey[2], *tval[2];
+    uint2 *pairs;        // [I] the binning's scattered (depth key, record) pairs
+    uint32_t *inst_rank; // [I] the binning's rank of each instance in its tile
+    uint32_t *sval;      // [I] records of the tile lists, in order
     float *slots;        // [I][9] adjoint slots (training workspaces only)
     float2 *imp_slots;   // [I] importance slots (alpha-weight, composited pixels as uint32 bits); a buffer
                          // of their own, so the importance sweep shares no scratch with the training pass
+                         // (the binning, which precedes both, merges its long lists there)
     // per tile
     uint2 *ranges;       // [T]
     // per pixel
@@ -395,9 +401,9 @@ struct gs_workspace {
     float *loss_partial; // [2 * blocks]
     size_t loss_partial_words;
     // scan / sort scratch
-    unsigned long long *lb_status; // preprocess: look-back + ticket of the gather and the projection
+    unsigned long long *lb_status; // preprocess: look-back + ticket of the gather and the projection (two words a chunk)
     size_t lb_words;
-    unsigned long long *bin_lb;    // binning: look-back + ticket of the count and the tile scan; zero between calls
+    unsigned long long *bin_lb;    // binning: look-back + ticket of the tile scan; zero between calls
     size_t bin_lb_words;
     uint32_t *rx_status; // radix: [4][256] histograms, then per pass [blocks * 256 + 1] look-back + ticket
     size_t rx_words;
@@ -446,7 +452,6 @@ struct gs_workspace {
     int have_binning;
     int have_compact;    // compact gradient rows of the current binning exist
     int imp_ready;       // the importance w, a of the current binning exist (gs_render_fwd_importance)
-    int tile_buf;        // buffer holding sorted instances (0)
     // kernel timing (gs_kernel_timing): event pairs around the rasterisers' launches
     static constexpr int kTimedPairs = 64;
     struct {

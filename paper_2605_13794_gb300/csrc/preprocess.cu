@@ -326,9 +326,13 @@ struct PreOut {
     uint32_t *gate_g;              // [N] block-strided candidates of the gate's first pass
     unsigned long long *gate_mask; // [N]
     const float *drift;            // [2][N] drift bounds (mean, log-scale) of deferred Adam steps, or NULL
-    unsigned long long *lb_status; // the projection's look-back, word 0: ticket (cleared by the gate)
+    uint32_t *inst_off, *chunk_rec;
+    // the projection's look-back over its chunks (cleared by the gate): word 0 the ticket, then the
+    // records of each chunk, then the instances
+    unsigned long long *lb_status, *lb_inst;
     DevCounters *ctr;
     long long max_records;
+    unsigned long long max_instances;
     const uint32_t *cull;
     long long cull_words;
 };
@@ -681,9 +685,13 @@ __device__ __forceinline__ RecOut make_record(const GaussPtrs &g, long long i, c
     return o;
 }
 
+// first: the record's first instance
 __device__ __forceinline__ void store_record(const PreOut &o, unsigned long long r, long long i, int c,
-                                             const RecOut &q)
+                                             const RecOut &q, unsigned long long first)
 {
+    o.inst_off[r] = (uint32_t)first;
+    const unsigned long long end = min(first + q.tt, o.max_instances);
+    for (unsigned long long m = (first + kBinChunk - 1) / kBinChunk; m * kBinChunk < end; m++) o.chunk_rec[m] = (uint32_t)r;
     o.rec_g[r] = (uint32_t)i;
     o.rec_cam[r] = (uint16_t)c;
     o.rd0[r] = q.rd0;
@@ -712,7 +720,7 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(GaussPtrs g, PreO
     __shared__ float s_thr2[kMaxLod + 1];
     __shared__ unsigned s_bid;
     __shared__ unsigned long long s_warp[kNW];
-    __shared__ unsigned long long s_base;
+    __shared__ unsigned long long s_base, s_ibase;
     const unsigned long long ncand = o.ctr->n_candidates;
     const int tw = ct.tile_w, th = ct.tile_h;
     if (threadIdx.x == 0) {
@@ -731,7 +739,7 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(GaussPtrs g, PreO
     GaussLoad L;
     L.have_shape = false;
     long long i = 0;
-    unsigned long long act = 0;
+    unsigned long long act = 0, tiles = 0; // active cameras, tiles of their records
     float op = 0.f;
     Proj p_one; // one camera: the projection of the active record
     if (j < ncand) {
@@ -751,6 +759,7 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(GaussPtrs g, PreO
             Proj p;
             if (project_gaussian(L.ls, L.q, td, s_cams[c], tw, th, rc, p)) {
                 act |= 1ull << c;
+                tiles += (unsigned)((p.x1 - p.x0) * (p.y1 - p.y0));
                 if (kOneCam) p_one = p;
             }
         }
@@ -764,12 +773,14 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(GaussPtrs g, PreO
             const int c = __ffsll((long long)mm) - 1;
             if (cull_bit(o, c, i)) marked |= 1ull << c;
         }
-    unsigned long long total;
+    unsigned long long total, itotal;
     const unsigned long long excl = block_exclusive_scan<kNW, unsigned long long>(cnt, s_warp, total);
+    const unsigned long long iexcl = block_exclusive_scan<kNW, unsigned long long>(tiles, s_warp, itotal);
     const int tvis = __syncthreads_count((act & ~marked) != 0);
-    // the chunk's count is published before the colours are read, so that no
+    // the chunk's counts are published before the colours are read, so that no
     // later chunk's look-back waits for them
     if (threadIdx.x == 0) lookback_publish(o.lb_status + 1, bid, total);
+    if (threadIdx.x == 32) lookback_publish(o.lb_inst, bid, itotal);
     RecOut one;
     if (kOneCam && act) one = make_record(g, i, L, op, s_cams[0], p_one, rc, marked & 1ull);
     if (threadIdx.x < 32) {
@@ -778,10 +789,14 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(GaussPtrs g, PreO
             s_base = b;
             if (tvis) atomicAdd(&o.ctr->n_visible, (unsigned long long)tvis); // the visible set of Eq. 5
         }
+    } else if (threadIdx.x < 64) {
+        const unsigned long long b = lookback_resolve(o.lb_inst, bid, itotal, o.ctr, kSitePreprocess);
+        if (threadIdx.x == 32) s_ibase = b;
     }
     __syncthreads();
-    const unsigned long long base = s_base + excl;
+    const unsigned long long base = s_base + excl, ibase = s_ibase + iexcl;
     if (j == ncand - 1) {
+        o.ctr->inst_total = ibase + tiles;
         const unsigned long long end = base + cnt;
         o.ctr->records_needed = end;
         o.ctr->n_records = end < (unsigned long long)o.max_records ? end : o.max_records;
@@ -789,9 +804,9 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(GaussPtrs g, PreO
     if (act) {
         if (kOneCam) {
             if (base >= (unsigned long long)o.max_records) set_error(o.ctr, GS_ERR_CAPACITY, kSitePreprocess);
-            else store_record(o, base, i, 0, one);
+            else store_record(o, base, i, 0, one, ibase);
         } else {
-            unsigned long long r = base;
+            unsigned long long r = base, first = ibase;
             for (unsigned long long mm = act; mm; mm &= mm - 1, r++) {
                 const int c = __ffsll((long long)mm) - 1;
                 if (r >= (unsigned long long)o.max_records) {
@@ -803,7 +818,9 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(GaussPtrs g, PreO
                 camera_point_df(L.m, cam, td);
                 Proj p;
                 project_gaussian(L.ls, L.q, td, cam, tw, th, rc, p); // same inputs: same (passing) result
-                store_record(o, r, i, c, make_record(g, i, L, op, cam, p, rc, (marked >> c) & 1ull));
+                const RecOut q = make_record(g, i, L, op, cam, p, rc, (marked >> c) & 1ull);
+                store_record(o, r, i, c, q, first);
+                first += q.tt;
             }
         }
     }
@@ -848,7 +865,7 @@ cudaError_t launch_preprocess(gs_workspace *ws, cudaStream_t st, const uint32_t 
     // look-back state (ticket in word 0 of each): the gather's, then the
     // projection's; the gate clears both
     const long long gather_words = (n + kGateChunk * kGatherChunks - 1) / (kGateChunk * kGatherChunks) + 1;
-    const long long lb_words = gather_words + pchunks + 1;
+    const long long lb_words = gather_words + 2 * (long long)pchunks + 1;
     if ((size_t)lb_words > ws->lb_words) return cudaErrorInvalidValue; // sized at creation
     PreOut o;
     o.rec_g = ws->rec_g; o.tt = ws->tt; o.dkey = ws->dkey;
@@ -857,6 +874,9 @@ cudaError_t launch_preprocess(gs_workspace *ws, cudaStream_t st, const uint32_t 
     o.gate_g = ws->gate_g; o.gate_mask = ws->gate_mask;
     o.drift = ws->lazy.enabled ? ws->lazy.drift : nullptr;
     o.lb_status = ws->lb_status + gather_words;
+    o.lb_inst = o.lb_status + 1 + pchunks;
+    o.inst_off = ws->inst_off; o.chunk_rec = ws->chunk_rec;
+    o.max_instances = (unsigned long long)ws->cap.max_instances;
     o.ctr = ws->ctr; o.max_records = ws->cap.max_records;
     o.cull = ws->rc.cull_enable ? cull : nullptr;
     o.cull_words = (n + 31) / 32;

@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(SquareShape<TW, TH>::threads)
 template <int TW, int TH> static void fwd_launch(gs_workspace *ws, cudaStream_t st, float *rgb, float *T_out)
 {
     launch_pdl(render_fwd_kernel<TW, TH>, ws->cams.total_tiles, SquareShape<TW, TH>::threads, 0, st,
-        ws->ranges, ws->tval[ws->tile_buf], ws->rd0, ws->rd1, ws->rd2, ws->d_cams, ws->rc, rgb, T_out, ws->T_final,
+        ws->ranges, ws->sval, ws->rd0, ws->rd1, ws->rd2, ws->d_cams, ws->rc, rgb, T_out, ws->T_final,
         ws->n_contrib, ws->tile_last);
 }
 
@@ -586,7 +586,7 @@ cudaError_t launch_render_bwd(gs_workspace *ws, cudaStream_t st, const float *dL
 {
     if (ws->cams.total_tiles == 0) return cudaSuccess;
     BwdRenderArgs a;
-    a.ranges = ws->ranges; a.vals = ws->tval[ws->tile_buf]; a.rd0 = ws->rd0; a.rd1 = ws->rd1; a.rd2 = ws->rd2;
+    a.ranges = ws->ranges; a.vals = ws->sval; a.rd0 = ws->rd0; a.rd1 = ws->rd1; a.rd2 = ws->rd2;
     a.inst_off = ws->inst_off; a.rect = ws->rect; a.T_final = ws->T_final; a.n_contrib = ws->n_contrib;
     a.tile_last = ws->tile_last;
     a.dL_drgb = dL_drgb; a.slots = ws->slots; a.ctr = ws->ctr;
@@ -817,7 +817,7 @@ template <bool FWD> static cudaError_t importance_launch(gs_workspace *ws, cudaS
 static ImpArgs importance_args(gs_workspace *ws)
 {
     ImpArgs a{};
-    a.ranges = ws->ranges; a.vals = ws->tval[ws->tile_buf]; a.rd0 = ws->rd0; a.rd1 = ws->rd1; a.rd2 = ws->rd2;
+    a.ranges = ws->ranges; a.vals = ws->sval; a.rd0 = ws->rd0; a.rd1 = ws->rd1; a.rd2 = ws->rd2;
     a.inst_off = ws->inst_off; a.rect = ws->rect; a.slots = ws->imp_slots; a.ctr = ws->ctr;
     return a;
 }
