@@ -103,7 +103,6 @@ struct DevCounters {
     unsigned long long instances_needed;
     unsigned long long inst_total;     // instances of the records (the projection's count)
     unsigned long long n_candidates;   // Gaussians passing the gate stage of preprocess
-    unsigned long long n_catchup;      // candidates behind the current Adam step (deferred steps to replay)
     int error;
     int error_site;
     unsigned long long sel_count[GS_MAX_CAMERAS]; // w > 0 entries per camera (importance)

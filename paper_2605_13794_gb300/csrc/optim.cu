@@ -568,61 +568,30 @@ struct LazyArgs {
 
 __device__ __forceinline__ int group_len(int k) { return k == 4 ? 48 : k == 3 ? 1 : k == 2 ? 4 : 3; }
 
-// The deferred steps run element-parallel.  A first kernel gives each
-// (Gaussian, parameter) pair one thread, which replays that parameter's missed
-// zero-gradient steps (and takes the gradient step): it reads last[i] and
-// never writes it, so the threads of one Gaussian need no ordering.  A second
-// kernel, one thread per Gaussian, then moves last[i] to the current step and
-// recomputes the drift bounds from the moments now stored.  Items: every
-// Gaussian (flush), the gate's candidates (catch-up, before projecting them) or
-// the Gaussians with a record (the gradient step).  A parameter whose m and v
-// are both +0 is a fixed point of the zero-gradient step (m and v stay +0, p
-// moves by (-lr m) / (sqrt(v) ibc2 + eps) = -0), so its replay is skipped and,
-// without a gradient step, it is not written at all.
+// The deferred steps run element-parallel, each value through its own missed
+// zero-gradient steps (and the gradient step).  Items: every Gaussian (flush),
+// the gate's candidates (catch-up, before projecting them) or the Gaussians
+// with a record (the gradient step).  A parameter whose m and v are both +0 is
+// a fixed point of the zero-gradient step (m and v stay +0, p moves by
+// (-lr m) / (sqrt(v) ibc2 + eps) = -0), so its replay is skipped and, without
+// a gradient step, it is not written at all.
 enum LazyMode { kLazyAll = 0, kLazyCandidates = 1, kLazyGrad = 2 };
-// kLazyCandidates runs over the list of the candidates that are behind (the
-// catch-up list), in the order a selection pass appended them: each
-// Gaussian's replay is independent of the others, so the order is immaterial.
 
 struct LazyItems {
-    const uint32_t *cand_g;    // kLazyCandidates: the catch-up list (Gaussians of the gate's candidates that are behind)
-    const uint32_t *rec_g;     // kLazyGrad: Gaussian of each record (a Gaussian's records contiguous)
+    const uint32_t *list;      // Gaussian of each item: the gate's candidates, or each record's (a Gaussian's contiguous)
     const float *cgrad;        // kLazyGrad: compact gradient rows at the first record
     const DevCounters *ctr;    // sizes of the device lists
-    long long n;               // kLazyAll: Gaussians
 };
 
-template <int MODE> __device__ __forceinline__ unsigned long long lazy_count(const LazyItems &it)
+// Parameter element idx of group k, from its step `from` to step t by
+// zero-gradient steps.
+__device__ __forceinline__ void lazy_param(const LazyArgs &a, int k, long long idx, int from, int t)
 {
-    return MODE == kLazyAll ? (unsigned long long)it.n
-                            : MODE == kLazyCandidates ? it.ctr->n_catchup : it.ctr->n_records;
-}
-
-// item j -> Gaussian i; false for a record that is not its Gaussian's first
-template <int MODE> __device__ __forceinline__ bool lazy_item(const LazyItems &it, unsigned long long j, long long &i)
-{
-    if (MODE == kLazyAll) { i = (long long)j; return true; }
-    if (MODE == kLazyCandidates) { i = it.cand_g[j]; return true; }
-    const uint32_t gi = it.rec_g[j];
-    if (j > 0 && it.rec_g[j - 1] == gi) return false;
-    i = gi;
-    return true;
-}
-
-// Parameter element idx of group k of Gaussian i: from its step `from` to step
-// t (kLazyGrad: the zero-gradient steps to t - 1, then the gradient step t).
-template <int MODE>
-__device__ __forceinline__ void lazy_param(const LazyArgs &a, int k, long long idx, int from, int t, float grad)
-{
-    const int to = MODE == kLazyGrad ? t - 1 : t;
     float mv = a.m[k][idx], vv = a.v[k][idx];
-    const bool zero = (__float_as_uint(mv) | __float_as_uint(vv)) == 0u;
-    if (zero && MODE != kLazyGrad) return;
+    if ((__float_as_uint(mv) | __float_as_uint(vv)) == 0u) return;
     float pv = a.p[k][idx];
-    if (!zero)
-        for (int s = from + 1; s <= to; s++)
-            adam_one(pv, 0.f, mv, vv, a.b1, a.b2, a.hist[10 * s + k], a.hist[10 * s + 5 + k], a.eps);
-    if (MODE == kLazyGrad) adam_one(pv, grad, mv, vv, a.b1, a.b2, a.hist[10 * t + k], a.hist[10 * t + 5 + k], a.eps);
+    for (int s = from + 1; s <= t; s++)
+        adam_one(pv, 0.f, mv, vv, a.b1, a.b2, a.hist[10 * s + k], a.hist[10 * s + 5 + k], a.eps);
     a.p[k][idx] = pv; a.m[k][idx] = mv; a.v[k][idx] = vv;
 }
 
@@ -665,7 +634,7 @@ __device__ __forceinline__ void lazy_all_group(const LazyArgs &a, int k, long lo
     // the last total % 4 elements
     for (unsigned long long e = chunks * 4 + blockIdx.x * 256ull + threadIdx.x; e < total; e += stride) {
         const int from = a.last[e / LEN];
-        if (from < t) lazy_param<kLazyAll>(a, k, (long long)e, from, t, 0.f);
+        if (from < t) lazy_param(a, k, (long long)e, from, t);
     }
 }
 
@@ -680,127 +649,131 @@ __global__ void __launch_bounds__(256) lazy_all_elem_kernel(LazyArgs a, long lon
     lazy_all_group<48>(a, 4, n, t);  // SH
 }
 
-// The Gaussians of a device list, 20 consecutive threads per Gaussian, one
-// per unit of its row: the 48 SH coefficients as 12 float4, the quaternion as
-// one float4 (both 16-byte aligned rows), and the 3 + 3 + 1 scalars of mean,
-// log-scale and opacity.  Every component takes exactly lazy_param's steps.
-// A record head j is its Gaussian's first record: its compact gradient row
-// is row j.
-constexpr int kLazyUnits = 20;
-__device__ __forceinline__ void lazy_unit(int u, int &k, int &el, int &row)
+// The drift bound of one group of three from its moments (mean: the sum over
+// the axes, log-scale: the largest), scaled by the step size at step t.
+__device__ __forceinline__ float lazy_drift(const LazyArgs &a, int k, int t, const float *mv, const float *vv)
 {
-    if (u < 12) { k = 4; el = 4 * u; row = 11 + el; }            // SH, float4
-    else if (u == 12) { k = 2; el = 0; row = 6; }                  // quaternion, float4
-    else if (u < 16) { k = 0; el = u - 13; row = el; }             // mean
-    else if (u < 19) { k = 1; el = u - 16; row = 3 + el; }         // log-scale
-    else { k = 3; el = 0; row = 10; }                              // opacity
-}
-
-// The gradient step of one unit (a float4 of SH or quaternion, or a scalar)
-// of Gaussian i: the zero-gradient steps it missed, then step t with its
-// gradient, exactly lazy_param's steps.  Every load it needs (last step,
-// p, m, v, gradient) is issued before any is used, so a unit waits for memory
-// once.
-__device__ __forceinline__ void lazy_grad_unit(const LazyArgs &a, const float *grad, long long i, int u, int k,
-                                               long long idx, int t)
-{
-    const int from = a.last[i];
-    if (u > 12) { // a scalar
-        float pv = a.p[k][idx], mv = a.m[k][idx], vv = a.v[k][idx];
-        const float g = grad[0];
-        if (from >= t) return;
-        if ((__float_as_uint(mv) | __float_as_uint(vv)) != 0u)
-            for (int s = from + 1; s <= t - 1; s++)
-                adam_one(pv, 0.f, mv, vv, a.b1, a.b2, a.hist[10 * s + k], a.hist[10 * s + 5 + k], a.eps);
-        adam_one(pv, g, mv, vv, a.b1, a.b2, a.hist[10 * t + k], a.hist[10 * t + 5 + k], a.eps);
-        a.p[k][idx] = pv; a.m[k][idx] = mv; a.v[k][idx] = vv;
-        return;
-    }
-    const float4 p4 = *reinterpret_cast<const float4 *>(a.p[k] + idx);
-    const float4 m4 = *reinterpret_cast<const float4 *>(a.m[k] + idx);
-    const float4 v4 = *reinterpret_cast<const float4 *>(a.v[k] + idx);
-    const float g[4] = {grad[0], grad[1], grad[2], grad[3]};
-    if (from >= t) return;
-    float pv[4] = {p4.x, p4.y, p4.z, p4.w}, mv[4] = {m4.x, m4.y, m4.z, m4.w}, vv[4] = {v4.x, v4.y, v4.z, v4.w};
+    float d = 0.f;
 #pragma unroll
-    for (int c = 0; c < 4; c++) {
-        if ((__float_as_uint(mv[c]) | __float_as_uint(vv[c])) != 0u)
-            for (int s = from + 1; s <= t - 1; s++)
-                adam_one(pv[c], 0.f, mv[c], vv[c], a.b1, a.b2, a.hist[10 * s + k], a.hist[10 * s + 5 + k], a.eps);
-        adam_one(pv[c], g[c], mv[c], vv[c], a.b1, a.b2, a.hist[10 * t + k], a.hist[10 * t + 5 + k], a.eps);
+    for (int l = 0; l < 3; l++) {
+        const float r = fabsf(mv[l]) / (sqrtf(vv[l]) + a.eps);
+        d = k == 0 ? d + r : fmaxf(d, r);
     }
-    *reinterpret_cast<float4 *>(a.p[k] + idx) = make_float4(pv[0], pv[1], pv[2], pv[3]);
-    *reinterpret_cast<float4 *>(a.m[k] + idx) = make_float4(mv[0], mv[1], mv[2], mv[3]);
-    *reinterpret_cast<float4 *>(a.v[k] + idx) = make_float4(vv[0], vv[1], vv[2], vv[3]);
+    return t > 0 ? a.drift_factor * a.hist[10 * t + k] * d : 0.f;
 }
 
-template <int MODE> __global__ void __launch_bounds__(256) lazy_list_vec_kernel(LazyArgs a, LazyItems it)
+// The Gaussians of a device list.  A warp reads its items (32 candidates, of
+// which few may be behind, or kLazyGradItems records, so that a single view's
+// records spread over all the warps) and the steps their values are current
+// at, and takes those that are behind two at a time, half a warp each: lanes 0 - 11 of a half the 48 SH coefficients as float4, lane
+// 12 the quaternion as float4 (both 16-byte aligned rows), lanes 13, 14 and 15
+// the mean, the log-scales and the opacity.  The lane of the mean and that of
+// the log-scales hold all the moments their drift bound needs, and the warp
+// moves last[] forward once its items are done, so no second pass reads the
+// moments again.  Bound by HBM and the latency of scattered rows (15 arrays):
+// on 1.15M Gaussians (8M in the model, eight views) the catch-up and the
+// gradient step take 454 + 702 us, where 20 threads per Gaussian, a selection
+// pass before and a pass for the bounds after each took 595 + 824.
+constexpr int kLazyGradItems = 8;
+template <int MODE> __global__ void __launch_bounds__(256, 4) lazy_list_kernel(LazyArgs a, LazyItems it)
 {
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
     const int t = *a.d_step;
-    const unsigned long long total = lazy_count<MODE>(it) * kLazyUnits;
-    for (unsigned long long e = blockIdx.x * 256ull + threadIdx.x; e < total; e += gridDim.x * 256ull) {
-        const unsigned long long j = e / kLazyUnits;
-        const int u = (int)(e - j * kLazyUnits);
-        long long i;
-        if (!lazy_item<MODE>(it, j, i)) continue;
-        int k, el, row;
-        lazy_unit(u, k, el, row);
-        const long long idx = i * group_len(k) + el;
-        if (MODE == kLazyGrad) {
-            lazy_grad_unit(a, it.cgrad + j * kGradRow + row, i, u, k, idx, t);
-            continue;
+    const unsigned long long total = MODE == kLazyGrad ? it.ctr->n_records : it.ctr->n_candidates;
+    const int lane = threadIdx.x & 31, u = lane & 15;
+    const int k = u < 12 ? 4 : u == 12 ? 2 : u == 13 ? 0 : u == 14 ? 1 : 3;
+    const int comps = u <= 12 ? 4 : u <= 14 ? 3 : 1, len = group_len(k), el = u < 12 ? 4 * u : 0;
+    const int row = u < 12 ? 11 + el : u == 12 ? 6 : u == 13 ? 0 : u == 14 ? 3 : 10; // in the gradient row
+    float *P = a.p[k], *M = a.m[k], *V = a.v[k];
+    constexpr int kItems = MODE == kLazyGrad ? kLazyGradItems : 32;
+    for (unsigned long long j0 = ((unsigned long long)blockIdx.x * 8 + (threadIdx.x >> 5)) * kItems; j0 < total;
+         j0 += gridDim.x * (8ull * kItems)) {
+        const unsigned long long j = j0 + lane;
+        uint32_t gi = 0;
+        int from = t;
+        if (lane < kItems && j < total) {
+            gi = it.list[j];
+            // a record that is not its Gaussian's first has no row
+            if (MODE == kLazyCandidates || j == 0 || it.list[j - 1] != gi) from = a.last[gi];
         }
-        const int from = a.last[i];
-        if (from >= t) continue;
-        // a catch-up (no gradient): only units with a moment that is not +0 move
-        if (u > 12) { // a scalar
-            lazy_param<MODE>(a, k, idx, from, t, 0.f);
-            continue;
-        }
-        const float4 m4 = *reinterpret_cast<const float4 *>(a.m[k] + idx);
-        const float4 v4 = *reinterpret_cast<const float4 *>(a.v[k] + idx);
-        float mv[4] = {m4.x, m4.y, m4.z, m4.w}, vv[4] = {v4.x, v4.y, v4.z, v4.w};
-        bool zero[4], any = false;
+        const bool behind = from < t;
+        for (unsigned rest = __ballot_sync(0xffffffffu, behind); rest;) {
+            const int s0 = __ffs(rest) - 1;
+            rest &= rest - 1u;
+            const int s1 = rest ? __ffs(rest) - 1 : s0;
+            const bool second = rest != 0u;
+            rest &= rest - 1u;
+            const int src = lane < 16 ? s0 : s1;
+            const long long i = __shfl_sync(0xffffffffu, gi, src);
+            const int f = __shfl_sync(0xffffffffu, from, src);
+            if (lane >= 16 && !second) continue;
+            const long long idx = i * len + el;
+            float pv[4] = {0.f, 0.f, 0.f, 0.f}, mv[4] = {0.f, 0.f, 0.f, 0.f}, vv[4] = {0.f, 0.f, 0.f, 0.f};
+            float g[4] = {0.f, 0.f, 0.f, 0.f};
+            // every load issued before any value is used
+            if (u <= 12) {
+                const float4 m4 = *reinterpret_cast<const float4 *>(M + idx), v4 = *reinterpret_cast<const float4 *>(V + idx);
+                mv[0] = m4.x; mv[1] = m4.y; mv[2] = m4.z; mv[3] = m4.w;
+                vv[0] = v4.x; vv[1] = v4.y; vv[2] = v4.z; vv[3] = v4.w;
+            } else {
 #pragma unroll
-        for (int c = 0; c < 4; c++) {
-            zero[c] = (__float_as_uint(mv[c]) | __float_as_uint(vv[c])) == 0u;
-            any = any || !zero[c];
-        }
-        if (!any) continue; // every component a fixed point
-        const float4 p4 = *reinterpret_cast<const float4 *>(a.p[k] + idx);
-        float pv[4] = {p4.x, p4.y, p4.z, p4.w};
+                for (int c = 0; c < 3; c++)
+                    if (c < comps) { mv[c] = M[idx + c]; vv[c] = V[idx + c]; }
+            }
+            if (MODE == kLazyGrad) {
+                const float *gr = it.cgrad + (j0 + src) * kGradRow + row;
 #pragma unroll
-        for (int c = 0; c < 4; c++) {
-            if (!zero[c])
-                for (int s2 = from + 1; s2 <= t; s2++)
-                    adam_one(pv[c], 0.f, mv[c], vv[c], a.b1, a.b2, a.hist[10 * s2 + k], a.hist[10 * s2 + 5 + k], a.eps);
+                for (int c = 0; c < 4; c++)
+                    if (c < comps) g[c] = gr[c];
+            }
+            unsigned moving = 0; // components with a moment that is not +0
+#pragma unroll
+            for (int c = 0; c < 4; c++) moving |= (__float_as_uint(mv[c]) | __float_as_uint(vv[c])) != 0u ? 1u << c : 0u;
+            if (MODE == kLazyGrad || moving) {
+                if (u <= 12) {
+                    const float4 p4 = *reinterpret_cast<const float4 *>(P + idx);
+                    pv[0] = p4.x; pv[1] = p4.y; pv[2] = p4.z; pv[3] = p4.w;
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 3; c++)
+                        if (c < comps) pv[c] = P[idx + c];
+                }
+                const int to = MODE == kLazyGrad ? t - 1 : t;
+#pragma unroll
+                for (int c = 0; c < 4; c++) {
+                    if ((moving >> c) & 1u)
+                        for (int s = f + 1; s <= to; s++)
+                            adam_one(pv[c], 0.f, mv[c], vv[c], a.b1, a.b2, a.hist[10 * s + k], a.hist[10 * s + 5 + k], a.eps);
+                    if (MODE == kLazyGrad && c < comps)
+                        adam_one(pv[c], g[c], mv[c], vv[c], a.b1, a.b2, a.hist[10 * t + k], a.hist[10 * t + 5 + k], a.eps);
+                }
+                if (u <= 12) {
+                    *reinterpret_cast<float4 *>(P + idx) = make_float4(pv[0], pv[1], pv[2], pv[3]);
+                    *reinterpret_cast<float4 *>(M + idx) = make_float4(mv[0], mv[1], mv[2], mv[3]);
+                    *reinterpret_cast<float4 *>(V + idx) = make_float4(vv[0], vv[1], vv[2], vv[3]);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 3; c++)
+                        if (c < comps) { P[idx + c] = pv[c]; M[idx + c] = mv[c]; V[idx + c] = vv[c]; }
+                }
+            }
+            if (u == 13) a.drift[i] = lazy_drift(a, 0, t, mv, vv);
+            if (u == 14) a.drift[a.n + i] = lazy_drift(a, 1, t, mv, vv);
         }
-        *reinterpret_cast<float4 *>(a.p[k] + idx) = make_float4(pv[0], pv[1], pv[2], pv[3]);
-        *reinterpret_cast<float4 *>(a.m[k] + idx) = make_float4(mv[0], mv[1], mv[2], mv[3]);
-        *reinterpret_cast<float4 *>(a.v[k] + idx) = make_float4(vv[0], vv[1], vv[2], vv[3]);
+        if (behind) a.last[gi] = t;
     }
 }
 
-// last[i] = t and the drift bounds of Gaussian i from its current moments
-template <int MODE> __global__ void __launch_bounds__(256) lazy_fin_kernel(LazyArgs a, LazyItems it)
+// last[i] = t and the drift bounds of every Gaussian from its current moments (after a flush)
+__global__ void __launch_bounds__(256) lazy_fin_kernel(LazyArgs a)
 {
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
     const int t = *a.d_step;
-    const unsigned long long cnt = lazy_count<MODE>(it);
-    for (unsigned long long j = blockIdx.x * 256ull + threadIdx.x; j < cnt; j += gridDim.x * 256ull) {
-        long long i;
-        if (!lazy_item<MODE>(it, j, i)) continue;
+    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < a.n; i += gridDim.x * 256ll) {
         if (a.last[i] >= t) continue;
         a.last[i] = t;
-        float dm = 0.f, ds = 0.f;
-#pragma unroll
-        for (int l = 0; l < 3; l++) {
-            dm += fabsf(a.m[0][3 * i + l]) / (sqrtf(a.v[0][3 * i + l]) + a.eps);
-            ds = fmaxf(ds, fabsf(a.m[1][3 * i + l]) / (sqrtf(a.v[1][3 * i + l]) + a.eps));
-        }
-        a.drift[i] = t > 0 ? a.drift_factor * a.hist[10 * t] * dm : 0.f;
-        a.drift[a.n + i] = t > 0 ? a.drift_factor * a.hist[10 * t + 1] * ds : 0.f;
+        a.drift[i] = lazy_drift(a, 0, t, a.m[0] + 3 * i, a.v[0] + 3 * i);
+        a.drift[a.n + i] = lazy_drift(a, 1, t, a.m[1] + 3 * i, a.v[1] + 3 * i);
     }
 }
 
@@ -832,14 +805,6 @@ static gs_gaussian_grads params_of(const gs_gaussians &g)
     return p;
 }
 
-static LazyItems lazy_items(gs_workspace *ws, long long n)
-{
-    LazyItems it;
-    it.cand_g = ws->cand_g; it.rec_g = ws->rec_g; it.cgrad = ws->cgrad;
-    it.ctr = ws->ctr; it.n = n;
-    return it;
-}
-
 // grid of up to 8 resident 256-thread blocks per SM, striding over `work` items
 static unsigned lazy_grid(gs_workspace *ws, unsigned long long work)
 {
@@ -847,60 +812,11 @@ static unsigned lazy_grid(gs_workspace *ws, unsigned long long work)
                                                                                    8ull * ws->sm_count));
 }
 
-template <int MODE>
-static cudaError_t launch_lazy_list(gs_workspace *ws, cudaStream_t st, const LazyArgs &a, unsigned long long cap)
-{
-    const LazyItems it = lazy_items(ws, 0);
-    if (MODE == kLazyGrad) kt_begin(ws, GS_KT_ADAM_GRAD, st);
-    launch_pdl(lazy_list_vec_kernel<MODE>, lazy_grid(ws, cap * kLazyUnits), 256, 0, st, a, it);
-    if (MODE == kLazyGrad) kt_end(ws, GS_KT_ADAM_GRAD, st);
-    note_launch();
-    launch_pdl(lazy_fin_kernel<MODE>, lazy_grid(ws, cap), 256, 0, st, a, it);
-    note_launch();
-    return cudaGetLastError();
-}
-
-// The catch-up list: the gate's candidates whose p, m, v are behind the
-// current step (in the steady state of a training run, few or none), appended
-// with one atomic per warp.
-__global__ void __launch_bounds__(256) lazy_select_kernel(const uint32_t *cand_g, const int32_t *last,
-                                                          const int *d_step, uint32_t *list, DevCounters *ctr)
-{
-    griddep_wait(); // programmatic dependent launch: the previous kernel is complete
-    const unsigned long long ncand = ctr->n_candidates;
-    const int t = *d_step, lane = threadIdx.x & 31;
-    for (unsigned long long j0 = (unsigned long long)blockIdx.x * 256 + (threadIdx.x & ~31u); j0 < ncand;
-         j0 += (unsigned long long)gridDim.x * 256) {
-        const unsigned long long j = j0 + lane;
-        uint32_t i = 0;
-        bool behind = false;
-        if (j < ncand) {
-            i = cand_g[j];
-            behind = last[i] < t;
-        }
-        const unsigned b = __ballot_sync(0xffffffffu, behind);
-        if (!b) continue;
-        unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(&ctr->n_catchup, (unsigned long long)__popc(b));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (behind) list[base + __popc(b & ((1u << lane) - 1u))] = i;
-    }
-}
-
 cudaError_t launch_lazy_catchup(gs_workspace *ws, cudaStream_t st, const gs_gaussians &g)
 {
     if (g.n == 0) return cudaSuccess;
-    // the list goes to the gate's per-chunk candidate buffer ([n], free once gathered)
-    launch_pdl(lazy_select_kernel, lazy_grid(ws, (unsigned long long)g.n), 256, 0, st, ws->cand_g, ws->lazy.last,
-               ws->d_adam_step, ws->gate_g, ws->ctr);
-    note_launch();
-    LazyArgs a = lazy_args(ws, params_of(g), g.n);
-    LazyItems it = lazy_items(ws, 0);
-    it.cand_g = ws->gate_g;
-    launch_pdl(lazy_list_vec_kernel<kLazyCandidates>, lazy_grid(ws, (unsigned long long)g.n * kLazyUnits), 256, 0,
-               st, a, it);
-    note_launch();
-    launch_pdl(lazy_fin_kernel<kLazyCandidates>, lazy_grid(ws, (unsigned long long)g.n), 256, 0, st, a, it);
+    launch_pdl(lazy_list_kernel<kLazyCandidates>, lazy_grid(ws, (unsigned long long)g.n), 256, 0, st,
+               lazy_args(ws, params_of(g), g.n), LazyItems{ws->cand_g, nullptr, ws->ctr});
     note_launch();
     return cudaGetLastError();
 }
@@ -911,7 +827,7 @@ cudaError_t launch_lazy_flush(gs_workspace *ws, cudaStream_t st, const gs_gaussi
     const LazyArgs a = lazy_args(ws, params_of(g), g.n);
     launch_pdl(lazy_all_elem_kernel, lazy_grid(ws, (unsigned long long)g.n * kGradRow), 256, 0, st, a, g.n);
     note_launch();
-    launch_pdl(lazy_fin_kernel<kLazyAll>, lazy_grid(ws, (unsigned long long)g.n), 256, 0, st, a, lazy_items(ws, g.n));
+    launch_pdl(lazy_fin_kernel, lazy_grid(ws, (unsigned long long)g.n), 256, 0, st, a);
     note_launch();
     return cudaGetLastError();
 }
@@ -919,7 +835,12 @@ cudaError_t launch_lazy_flush(gs_workspace *ws, cudaStream_t st, const gs_gaussi
 static cudaError_t launch_lazy_adam(gs_workspace *ws, cudaStream_t st, const gs_gaussian_grads &param, long long n)
 {
     if (ws->cap.max_records == 0) return cudaSuccess;
-    return launch_lazy_list<kLazyGrad>(ws, st, lazy_args(ws, param, n), (unsigned long long)ws->cap.max_records);
+    kt_begin(ws, GS_KT_ADAM_GRAD, st);
+    launch_pdl(lazy_list_kernel<kLazyGrad>, lazy_grid(ws, (unsigned long long)ws->cap.max_records * (32 / kLazyGradItems)), 256, 0, st,
+               lazy_args(ws, param, n), LazyItems{ws->rec_g, ws->cgrad, ws->ctr});
+    kt_end(ws, GS_KT_ADAM_GRAD, st);
+    note_launch();
+    return cudaGetLastError();
 }
 
 // First record of each Gaussian with records, for the dense pass's lookups.
