@@ -47,7 +47,7 @@ struct Layout {
 
 struct Offsets {
     size_t cand_g, cand_mask, gate_cnt, gate_g, gate_mask, rec_first, cgrad, rec_g, rec_cam, rd0, rd1, rd2, rect, tt, inst_off, chunk_rec, clampm, rgrad, dkey, tile_cnt, tile_last;
-    size_t pairs, inst_rank, sval, slots, imp_slots, ranges, n_contrib, T_final, imp_w, imp_a, sel_cum, sel_bsum;
+    size_t pairs, inst_rank, sval, visits, slots, imp_slots, ranges, n_contrib, T_final, imp_w, imp_a, sel_cum, sel_bsum;
     size_t selk0, selk1, selv0, selv1, loss_maps, loss_partial, lb_status, bin_lb, rx_status, red_partial,
         ctr, d_cams, d_adam_step, d_adam_coef;
     size_t mkey0, mkey1, mval0, mval1, mcum, mbsum, mrx_status, mlb, mhist, mctr;
@@ -84,6 +84,7 @@ Offsets plan(const gs_capacity &c)
     o.pairs = L.take<uint2>(I);
     o.inst_rank = L.take<uint32_t>(I);
     o.sval = L.take<uint32_t>(I);
+    o.visits = L.take<uint32_t>(fwd_only ? 0 : (I / 32 + T) * 8); // at most eight warps (32 x 16 pixels) per tile
     o.slots = L.take<float>(fwd_only ? 0 : I * gs::kSlotFloats);
     o.imp_slots = L.take<float2>(I); // importance (w, a) per instance
     o.ranges = L.take<uint2>(T);
@@ -286,6 +287,7 @@ int gs_workspace_create(const gs_capacity *cap, gs_workspace **out)
     ws->pairs = (uint2 *)(b + o.pairs);
     ws->inst_rank = (uint32_t *)(b + o.inst_rank);
     ws->sval = (uint32_t *)(b + o.sval);
+    ws->visits = (cap->flags & GS_CAP_FORWARD_ONLY) ? nullptr : (uint32_t *)(b + o.visits);
     ws->slots = (float *)(b + o.slots);
     ws->imp_slots = (float2 *)(b + o.imp_slots);
     ws->ranges = (uint2 *)(b + o.ranges);

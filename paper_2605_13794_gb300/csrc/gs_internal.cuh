@@ -384,6 +384,8 @@ struct gs_workspace {
     float2 *imp_slots;   // [I] importance slots (alpha-weight, composited pixels as uint32 bits); a buffer
                          // of their own, so the importance sweep shares no scratch with the training pass
                          // (the binning, which precedes both, merges its long lists there)
+    uint32_t *visits;    // [I / 32 + T][warps of a tile] entries of each batch that composite in each warp's
+                         // square (forward -> adjoint; NULL in a forward-only workspace)
     // per tile
     uint2 *ranges;       // [T]
     // per pixel

@@ -219,6 +219,21 @@ __device__ __forceinline__ float2 pair_power(float4 e0, float Ds, float2 pxc, fl
     return __ffma2_rn(f2(e0.z), __fmul2_rn(e, e), f2(ddy));
 }
 
+// The entries of a batch (list positions b .. b + 31 of the tile whose list
+// starts at start) that composite in a warp's square, one bit each, left by the
+// forward for the adjoint.  Tiles' batches follow one another, each tile's from
+// start / 32 + its index.
+template <int WARPS> __device__ __forceinline__ size_t visits_at(int start, int b, int warp)
+{
+    return ((size_t)(start / 32) + blockIdx.x + (unsigned)(b - start) / 32u) * WARPS + warp;
+}
+template <int WARPS>
+__device__ __forceinline__ void put_visits(uint32_t *visits, int start, int b, int warp, unsigned comp)
+{
+    comp = __reduce_or_sync(0xffffffffu, comp);
+    if ((threadIdx.x & 31) == 0) visits[visits_at<WARPS>(start, b, warp)] = comp;
+}
+
 // ---- forward --------------------------------------------------------------
 //
 // Front to back over the visited entries of each batch; a warp stops once all
@@ -227,13 +242,15 @@ __device__ __forceinline__ float2 pair_power(float4 e0, float Ds, float2 pxc, fl
 // saved (24 mixed views, whole pass: 2.84 ms with it, 2.79 without), as did a
 // vote to skip the entries that reach no live pixel (3.06 ms).
 
-template <int TW, int TH>
+// VISITS: note the entries that composite in each square for the adjoint (not in
+// a forward-only workspace: the bookkeeping costs the walk 6 %).
+template <int TW, int TH, bool VISITS>
 __global__ void __launch_bounds__(SquareShape<TW, TH>::threads)
     render_fwd_kernel(const uint2 *__restrict__ ranges, const uint32_t *__restrict__ vals,
                       const float4 *__restrict__ rd0, const float4 *__restrict__ rd1, const float4 *__restrict__ rd2,
                       const CamTable *__restrict__ ctp, RenderConsts rc, float *__restrict__ rgb_out,
                       float *__restrict__ T_out, float *__restrict__ T_ws, uint32_t *__restrict__ n_contrib,
-                      uint32_t *__restrict__ tile_last)
+                      uint32_t *__restrict__ tile_last, uint32_t *__restrict__ visits)
 {
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
     constexpr int kWarps = SquareShape<TW, TH>::warps;
@@ -266,6 +283,7 @@ __global__ void __launch_bounds__(SquareShape<TW, TH>::threads)
         }
         unsigned m = __ballot_sync(0xffffffffu, visit);
         __syncwarp();
+        unsigned comp = 0; // entries that composite in the lane's pixels
         while (m != 0u) {
             const int jj = __ffs(m) - 1; // front to back
             m &= m - 1u;
@@ -283,6 +301,7 @@ __global__ void __launch_bounds__(SquareShape<TW, TH>::threads)
             const bool c0 = ok0 && !st0, c1 = ok1 && !st1;
             dn0 = dn0 || st0;
             dn1 = dn1 || st1;
+            if (VISITS && (c0 || c1)) comp |= 1u << jj;
             const float2 ae = make_float2(c0 ? al.x : 0.f, c1 ? al.y : 0.f); // skipped fragments add nothing
             const float2 w = __fmul2_rn(ae, T);
             Cr = __ffma2_rn(w, f2(p1.z), Cr);
@@ -292,6 +311,7 @@ __global__ void __launch_bounds__(SquareShape<TW, TH>::threads)
             last0 = c0 ? pos : last0;
             last1 = c1 ? pos : last1;
         }
+        if (VISITS) put_visits<kWarps>(visits, start, b, warp, comp);
         __syncwarp();
     }
     const long long np = (long long)cam.width * cam.height;
@@ -316,9 +336,10 @@ __global__ void __launch_bounds__(SquareShape<TW, TH>::threads)
 
 template <int TW, int TH> static void fwd_launch(gs_workspace *ws, cudaStream_t st, float *rgb, float *T_out)
 {
-    launch_pdl(render_fwd_kernel<TW, TH>, ws->cams.total_tiles, SquareShape<TW, TH>::threads, 0, st,
+    const auto kernel = ws->visits ? render_fwd_kernel<TW, TH, true> : render_fwd_kernel<TW, TH, false>;
+    launch_pdl(kernel, ws->cams.total_tiles, SquareShape<TW, TH>::threads, 0, st,
         ws->ranges, ws->sval, ws->rd0, ws->rd1, ws->rd2, ws->d_cams, ws->rc, rgb, T_out, ws->T_final,
-        ws->n_contrib, ws->tile_last);
+        ws->n_contrib, ws->tile_last, ws->visits);
 }
 
 cudaError_t launch_render_fwd(gs_workspace *ws, cudaStream_t st, float *rgb, float *T_out)
@@ -343,14 +364,14 @@ cudaError_t launch_render_fwd(gs_workspace *ws, cudaStream_t st, float *rgb, flo
 //
 // Each warp owns an 8 x 8 pixel square of the tile -- lane l the horizontal
 // pixel pair (2 (l % 4), l / 4) of it, packed as FP32x2 -- and walks the
-// tile's list back to front on its own, in batches that start at the tile's
-// last contribution (the forward's largest n_contrib of the tile), visiting
-// only entries in front of its own pixels' last contribution and recovering T
-// by T / (1 - alpha) from the final transmittance.  It stages each batch of 32
-// entries itself (one per lane), so no block-wide barrier holds it while
-// another warp of the tile has more to do; the staging lane also tests its
-// entry's alpha footprint against the warp's square, and one ballot gives the
-// batch's entries the warp must visit.  Per visited entry the warp's nine slot
+// tile's list back to front on its own, in the forward's batches, starting with
+// the batch of the tile's last contribution (the forward's largest n_contrib of
+// the tile) and recovering T by T / (1 - alpha) from the final transmittance.
+// It visits exactly the entries that composite in its square, which the forward
+// noted (visits), so it tests no footprint, gathers only those entries' records
+// and needs no vote per visit.  It stages its entries itself (one per lane), so
+// no block-wide barrier holds it while another warp of the tile has more to do.
+// Per visited entry the warp's nine slot
 // values are one warp reduction; the warps' partials of a batch are summed in
 // warp order by the warp that finishes that batch last (shared-memory arrival
 // counters) and written to the entries' slots.  A warp may run up to
@@ -370,6 +391,7 @@ struct BwdRenderArgs {
     const float *T_final;
     const uint32_t *n_contrib;
     const uint32_t *tile_last; // largest n_contrib of each tile (the forward's)
+    const uint32_t *visits;    // entries of each batch that composite in each warp's square (the forward's)
     const float *dL_drgb;
     float *slots;
     DevCounters *ctr; // fragments += sum of the tile's n_contrib; composited += composited pairs
@@ -384,7 +406,6 @@ __global__ void __launch_bounds__(SquareShape<TW, TH>::threads, SquareShape<TW, 
     __shared__ float4 s0[kWarps][kBwdBatch];
     __shared__ float4 s1[kWarps][kBwdBatch];
     __shared__ float s2[kWarps][kBwdBatch];
-    __shared__ unsigned long long s_slot[kWarps][kBwdBatch];
     __shared__ float s_part[kBwdBufs][kWarps][kBwdBatch][kSlotFloats];
     __shared__ unsigned s_mask[kBwdBufs][kWarps]; // entries of the batch each warp visited
     __shared__ int s_arrive[kBwdBufs], s_done[kBwdBufs];
@@ -397,9 +418,9 @@ __global__ void __launch_bounds__(SquareShape<TW, TH>::threads, SquareShape<TW, 
     const float ox = (float)(tx * TW), oy = (float)(ty * TH);
     const uint2 rg = a.ranges[blockIdx.x];
     const int start = (int)rg.x, end = (int)rg.y;
-    // the reverse walk starts after the tile's last contribution (the forward's
-    // largest n_contrib); entries behind it carry zero gradient
-    const int last = start + min((int)a.tile_last[blockIdx.x], end - start);
+    // the reverse walk starts with the batch of the tile's last contribution
+    // (the forward's largest n_contrib); entries behind it carry zero gradient
+    const int batches = (min((int)a.tile_last[blockIdx.x], end - start) + kBwdBatch - 1) / kBwdBatch;
     if (threadIdx.x < kBwdBufs) { s_arrive[threadIdx.x] = 0; s_done[threadIdx.x] = 0; }
     __syncthreads(); // the only block barrier: the arrival counters are set
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -410,7 +431,6 @@ __global__ void __launch_bounds__(SquareShape<TW, TH>::threads, SquareShape<TW, 
     const int lx = sx + 2 * (lane & 3), ly = sy + (lane >> 2);
     const float2 pxc = make_float2((float)lx + 0.5f, (float)lx + 1.5f);
     const float pyc = (float)ly + 0.5f;
-    const float bx0 = (float)sx + 0.5f, bx1 = (float)sx + 7.5f, by0 = (float)sy + 0.5f, by1 = (float)sy + 7.5f;
 
     // per-pixel state of the pair: dL/dC (g), T (from T_final back to each
     // fragment's own), S = colour composited behind the current fragment plus
@@ -444,25 +464,18 @@ __global__ void __launch_bounds__(SquareShape<TW, TH>::threads, SquareShape<TW, 
     }
     int ncomp = 0;
     int b = 0;
-    for (int hi = last; hi > start; hi -= kBwdBatch, b++) {
-        const int lo = max(start, hi - kBwdBatch);
-        const int cnt = hi - lo;
+    for (int lo = start + (batches - 1) * kBwdBatch; lo >= start; lo -= kBwdBatch, b++) {
+        const int cnt = min(kBwdBatch, end - lo);
         const int buf = b % kBwdBufs;
-        bool visit = false;
-        if (lane < cnt) {
-            const uint32_t r = a.vals[lo + lane];
+        // (a batch behind the warp's own last contribution may not have been walked by the forward)
+        const unsigned vmask = lo - start < wmax ? a.visits[visits_at<kWarps>(start, lo, warp)] : 0u;
+        const uint32_t r = lane < cnt ? a.vals[lo + lane] : 0u;
+        if ((vmask >> lane) & 1u) {
             const float4 r0 = a.rd0[r], r1 = a.rd1[r], r2 = a.rd2[r];
-            const float op = r2.w != 0.f ? 0.f : r1.y; // a record marked culled composites nowhere
-            const float4 e0 = stage_e0_at(r0, r2, ox, oy);
-            s0[warp][lane] = e0;
-            s1[warp][lane] = make_float4(stage_D(r1), op, r1.z, r1.w);
+            s0[warp][lane] = stage_e0_at(r0, r2, ox, oy);
+            s1[warp][lane] = make_float4(stage_D(r1), r1.y, r1.z, r1.w);
             s2[warp][lane] = r2.x;
-            s_slot[warp][lane] = slot_of(a.inst_off, a.rect, r, tx, ty);
-            // visited: in front of the warp's last contribution, alpha footprint meeting the square
-            visit = lo + lane - start < wmax &&
-                    square_visit(r0.z, r0.w, r1.x, op, rc.alpha_min, e0.x, e0.y, bx0, bx1, by0, by1);
         }
-        const unsigned vmask = __ballot_sync(0xffffffffu, visit);
         // the partial buffer of this batch is free once batch b - kBwdBufs has been summed
         if (b >= kBwdBufs) {
             const int want = b / kBwdBufs;
@@ -496,48 +509,45 @@ __global__ void __launch_bounds__(SquareShape<TW, TH>::threads, SquareShape<TW, 
             // composited pixels: in front of the pixel's last contribution, alpha >= alpha_min
             const bool m0 = j < nc0 && al.x >= rc.alpha_min;
             const bool m1 = j < nc1 && al.y >= rc.alpha_min;
-            float r = 0.f;
-            if (__any_sync(0xffffffffu, m0 || m1)) {
-                // Every lane runs the adjoint (no divergent branch): a pixel that does not
-                // composite here has aT = dG = 0, so it adds exact zeros and keeps its T and S
-                // (all terms stay finite: alpha <= alpha_max < 1).
-                ncomp += (int)m0 + (int)m1;
-                const float cb = s2[warp][jj];
-                const float2 inv = make_float2(rcp_approx(1.f - al.x), rcp_approx(1.f - al.y));
-                const float2 Tj = __fmul2_rn(T, inv); // transmittance in front of this fragment
-                const float2 aTf = __fmul2_rn(al, Tj);
-                const float2 aT = make_float2(m0 ? aTf.x : 0.f, m1 ? aTf.y : 0.f);
-                // dL/dalpha = Tj (g . c) - (g . S) / (1 - alpha)
-                const float2 gc = __ffma2_rn(g2, f2(cb), __ffma2_rn(g1, f2(p1.w), __fmul2_rn(g0, f2(p1.z))));
-                const float2 gS = __ffma2_rn(g2, S2, __ffma2_rn(g1, S1, __fmul2_rn(g0, S0)));
-                const float2 dal = __ffma2_rn(make_float2(-inv.x, -inv.y), gS, __fmul2_rn(Tj, gc));
-                S0 = __ffma2_rn(aT, f2(p1.z), S0);
-                S1 = __ffma2_rn(aT, f2(p1.w), S1);
-                S2 = __ffma2_rn(aT, f2(cb), S2);
-                T = make_float2(m0 ? Tj.x : T.x, m1 ? Tj.y : T.y);
-                // dL/do of the pixel = G dL/dalpha, zero where alpha is clamped at alpha_max;
-                // dL/dpower = o times it
-                const float2 dGf = __fmul2_rn(G, dal);
-                const float2 dG = make_float2(m0 && al.x < rc.alpha_max ? dGf.x : 0.f,
-                                              m1 && al.y < rc.alpha_max ? dGf.y : 0.f);
-                // The slot takes dG-weighted moments of the pixel offsets: the record's
-                // opacity and conic factors of the mean and conic gradients are applied
-                // once per record, when its slots are summed (slot_grads_from_moments).
-                float v[kSlotFloats];
-                const float sG = dG.x + dG.y;
-                const float2 gx = __fmul2_rn(dG, dx);
-                v[0] = fmaf(dG.y, e.y, dG.x * e.x);   // sum dG e,  e = dx + k dy
-                v[1] = sG * dy;                       // sum dG dy
-                v[2] = fmaf(gx.y, dx.y, gx.x * dx.x); // sum dG dx^2
-                v[3] = (gx.x + gx.y) * dy;            // sum dG dx dy
-                v[4] = v[1] * dy;                     // sum dG dy^2
-                v[5] = sG;                            // dL/do = sum dG
-                v[6] = fmaf(aT.y, g0.y, aT.x * g0.x); // dL/dc = sum alpha T dL/dC
-                v[7] = fmaf(aT.y, g1.y, aT.x * g1.x);
-                v[8] = fmaf(aT.y, g2.y, aT.x * g2.x);
-                r = warp_reduce9(v, lane);
-            }
-            if (red_own) part[jj][red_q] = r;
+            // Every lane runs the adjoint (no divergent branch): a pixel that does not
+            // composite here has aT = dG = 0, so it adds exact zeros and keeps its T and S
+            // (all terms stay finite: alpha <= alpha_max < 1).
+            ncomp += (int)m0 + (int)m1;
+            const float cb = s2[warp][jj];
+            const float2 inv = make_float2(rcp_approx(1.f - al.x), rcp_approx(1.f - al.y));
+            const float2 Tj = __fmul2_rn(T, inv); // transmittance in front of this fragment
+            const float2 aTf = __fmul2_rn(al, Tj);
+            const float2 aT = make_float2(m0 ? aTf.x : 0.f, m1 ? aTf.y : 0.f);
+            // dL/dalpha = Tj (g . c) - (g . S) / (1 - alpha)
+            const float2 gc = __ffma2_rn(g2, f2(cb), __ffma2_rn(g1, f2(p1.w), __fmul2_rn(g0, f2(p1.z))));
+            const float2 gS = __ffma2_rn(g2, S2, __ffma2_rn(g1, S1, __fmul2_rn(g0, S0)));
+            const float2 dal = __ffma2_rn(make_float2(-inv.x, -inv.y), gS, __fmul2_rn(Tj, gc));
+            S0 = __ffma2_rn(aT, f2(p1.z), S0);
+            S1 = __ffma2_rn(aT, f2(p1.w), S1);
+            S2 = __ffma2_rn(aT, f2(cb), S2);
+            T = make_float2(m0 ? Tj.x : T.x, m1 ? Tj.y : T.y);
+            // dL/do of the pixel = G dL/dalpha, zero where alpha is clamped at alpha_max;
+            // dL/dpower = o times it
+            const float2 dGf = __fmul2_rn(G, dal);
+            const float2 dG = make_float2(m0 && al.x < rc.alpha_max ? dGf.x : 0.f,
+                                          m1 && al.y < rc.alpha_max ? dGf.y : 0.f);
+            // The slot takes dG-weighted moments of the pixel offsets: the record's
+            // opacity and conic factors of the mean and conic gradients are applied
+            // once per record, when its slots are summed (slot_grads_from_moments).
+            float v[kSlotFloats];
+            const float sG = dG.x + dG.y;
+            const float2 gx = __fmul2_rn(dG, dx);
+            v[0] = fmaf(dG.y, e.y, dG.x * e.x);   // sum dG e,  e = dx + k dy
+            v[1] = sG * dy;                       // sum dG dy
+            v[2] = fmaf(gx.y, dx.y, gx.x * dx.x); // sum dG dx^2
+            v[3] = (gx.x + gx.y) * dy;            // sum dG dx dy
+            v[4] = v[1] * dy;                     // sum dG dy^2
+            v[5] = sG;                            // dL/do = sum dG
+            v[6] = fmaf(aT.y, g0.y, aT.x * g0.x); // dL/dc = sum alpha T dL/dC
+            v[7] = fmaf(aT.y, g1.y, aT.x * g1.x);
+            v[8] = fmaf(aT.y, g2.y, aT.x * g2.x);
+            const float sum = warp_reduce9(v, lane);
+            if (red_own) part[jj][red_q] = sum;
         }
         // arrive; the last warp of the tile to finish this batch sums it
         __syncwarp();
@@ -561,7 +571,7 @@ __global__ void __launch_bounds__(SquareShape<TW, TH>::threads, SquareShape<TW, 
                         for (int q = 0; q < kSlotFloats; q++) sum[q] += s_part[buf][w][lane][q];
                     }
                 }
-                float *dst = a.slots + s_slot[warp][lane] * kSlotFloats;
+                float *dst = a.slots + slot_of(a.inst_off, a.rect, r, tx, ty) * kSlotFloats;
 #pragma unroll
                 for (int q = 0; q < kSlotFloats; q++) dst[q] = sum[q];
             }
@@ -573,8 +583,8 @@ __global__ void __launch_bounds__(SquareShape<TW, TH>::threads, SquareShape<TW, 
             }
         }
     }
-    // entries after the tile's last contribution carry zero gradient
-    for (int s = last + threadIdx.x; s < end; s += kRT) {
+    // entries after the batch of the tile's last contribution carry zero gradient
+    for (int s = start + batches * kBwdBatch + threadIdx.x; s < end; s += kRT) {
         float *dst = a.slots + slot_of(a.inst_off, a.rect, a.vals[s], tx, ty) * kSlotFloats;
 #pragma unroll
         for (int k = 0; k < kSlotFloats; k++) dst[k] = 0.f;
@@ -590,6 +600,7 @@ cudaError_t launch_render_bwd(gs_workspace *ws, cudaStream_t st, const float *dL
     a.ranges = ws->ranges; a.vals = ws->sval; a.rd0 = ws->rd0; a.rd1 = ws->rd1; a.rd2 = ws->rd2;
     a.inst_off = ws->inst_off; a.rect = ws->rect; a.T_final = ws->T_final; a.n_contrib = ws->n_contrib;
     a.tile_last = ws->tile_last;
+    a.visits = ws->visits;
     a.dL_drgb = dL_drgb; a.slots = ws->slots; a.ctr = ws->ctr;
     const unsigned grid = (unsigned)ws->cams.total_tiles;
     kt_begin(ws, GS_KT_RENDER_BWD, st);
@@ -635,6 +646,7 @@ struct ImpArgs {
     float *rgb_out, *T_out, *T_ws;
     uint32_t *n_contrib;
     uint32_t *tile_last;   // the tile's largest n_contrib (atomic max; zeroed by the binning)
+    uint32_t *visits;      // as render_fwd_kernel's, or NULL
 };
 
 template <int TW, int TH, bool FWD>
@@ -703,6 +715,7 @@ __global__ void __launch_bounds__(SquareShape<TW, TH>::threads, SquareShape<TW, 
         }
         __syncwarp();
         if (lane == 0) s_mask[buf][warp] = vmask;
+        unsigned comp = 0; // FWD: entries that composite in the lane's pixels of the image
         for (unsigned m = vmask; m != 0u;) {
             const int jj = __ffs(m) - 1; // front to back
             m &= m - 1u;
@@ -721,6 +734,7 @@ __global__ void __launch_bounds__(SquareShape<TW, TH>::threads, SquareShape<TW, 
                 const bool c0 = ok0 && !st0, c1 = ok1 && !st1;
                 dn0 = dn0 || st0;
                 dn1 = dn1 || st1;
+                if (c0 || c1) comp |= 1u << jj;
                 const float2 ae = make_float2(c0 ? al.x : 0.f, c1 ? al.y : 0.f);
                 const float2 w = __fmul2_rn(ae, T);
                 const float2 rgc = s3[FWD ? warp : 0][jj];
@@ -749,6 +763,7 @@ __global__ void __launch_bounds__(SquareShape<TW, TH>::threads, SquareShape<TW, 
             }
             if (lane == 0) s_part[buf][warp][jj] = make_float2(wv, __uint_as_float(av));
         }
+        if (FWD && a.visits && !wdone) put_visits<kWarps>(a.visits, start, b, warp, comp);
         // arrive; the last warp of the tile to finish this batch sums it
         __syncwarp();
         int arrived = 0;
@@ -839,6 +854,7 @@ cudaError_t launch_render_fwd_importance(gs_workspace *ws, cudaStream_t st, floa
     if (ws->cams.total_tiles == 0) return cudaSuccess;
     ImpArgs a = importance_args(ws);
     a.rgb_out = rgb; a.T_out = T_out; a.T_ws = ws->T_final; a.n_contrib = ws->n_contrib; a.tile_last = ws->tile_last;
+    a.visits = ws->visits;
     kt_begin(ws, GS_KT_RENDER_FWD, st);
     cudaError_t e = importance_launch<true>(ws, st, a);
     if (e != cudaSuccess) return e;
