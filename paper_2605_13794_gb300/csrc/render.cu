@@ -57,8 +57,8 @@ __device__ __forceinline__ float2 pair_alpha(float2 p, float o, float amax, floa
 }
 
 // Whether an entry can composite anywhere in a warp's square, the box
-// [bx0, bx1] x [by0, by1] of its pixel centres (tile-local; (u, v) the entry's
-// tile-local mean).  alpha >= alpha_min needs o G >= alpha_min, i.e.
+// [bx0, bx0 + 7] x [by0, by0 + 7] of its pixel centres (tile-local; (u, v) the
+// entry's tile-local mean).  alpha >= alpha_min needs o G >= alpha_min, i.e.
 // q = A (dx + k dy)^2 + D dy^2 <= tau, tau = 2 ln(o / alpha_min).  The test
 // compares tau with the minimum of q over the box.  q is convex with its
 // minimum 0 at the mean, so on the way from any point of the box towards the
@@ -70,27 +70,32 @@ __device__ __forceinline__ float2 pair_alpha(float2 p, float o, float amax, floa
 // Widened (tau by 0.2 % + 2e-3, the box by 1/32 px) far beyond the FP32 error
 // of the exponent the kernels evaluate and of the approximate logarithm and
 // reciprocal here (a few units in the last place), so no pixel of a square that
-// fails can reach alpha_min in them; false when o is below alpha_min.
+// fails can reach alpha_min in them; it always fails when o is below alpha_min.
 // A warp skips an entry that fails: it composites nowhere in the warp, so
 // skipping it changes nothing.  (The bounding box of the ellipse and a looser
 // bound of q, before, took as many instructions and dropped fewer: the eight-view
 // training step of 8M Gaussians 7.68 ms with them, 7.61 with this test.)
-__device__ __forceinline__ bool square_visit(float A, float k, float D, float o, float alpha_min, float u, float v,
-                                             float bx0, float bx1, float by0, float by1)
-{
-    float tau = 2.f * __logf(__fdividef(o, alpha_min));
-    tau = fmaf(tau, 1.002f, 2e-3f);
-    if (!(tau > 0.f)) return false;
-    const float dx0 = bx0 - 0.03125f - u, dx1 = bx1 + 0.03125f - u, dy0 = by0 - 0.03125f - v, dy1 = by1 + 0.03125f - v;
-    const float xe = fminf(fmaxf(0.f, dx0), dx1), ye = fminf(fmaxf(0.f, dy0), dy1);
-    const float Ak = A * k;
-    const float y1 = fminf(fmaxf(-Ak * xe * rcp_approx(fmaf(Ak, k, D)), dy0), dy1);
-    const float s1 = fmaf(k, y1, xe);
-    const float x2 = fminf(fmaxf(-k * ye, dx0), dx1);
-    const float s2 = fmaf(k, ye, x2);
-    const float q = fminf(fmaf(A * s1, s1, D * y1 * y1), fmaf(A * s2, s2, D * ye * ye));
-    return !(q > tau);
-}
+struct SquareTest {
+    float A, k, D, tau, slope, u, v;
+    __device__ __forceinline__ SquareTest(float4 r0, float D_, float o, float alpha_min, float u_, float v_)
+        : A(r0.z), k(r0.w), D(D_), u(u_), v(v_)
+    {
+        tau = fmaf(2.f * __logf(__fdividef(o, alpha_min)), 1.002f, 2e-3f);
+        slope = -A * k * rcp_approx(fmaf(A * k, k, D));
+    }
+    __device__ __forceinline__ bool meets(float bx0, float by0) const
+    {
+        const float dx0 = bx0 - 0.03125f - u, dx1 = bx0 + 7.03125f - u;
+        const float dy0 = by0 - 0.03125f - v, dy1 = by0 + 7.03125f - v;
+        const float xe = fminf(fmaxf(0.f, dx0), dx1), ye = fminf(fmaxf(0.f, dy0), dy1);
+        const float y1 = fminf(fmaxf(slope * xe, dy0), dy1);
+        const float s1 = fmaf(k, y1, xe);
+        const float x2 = fminf(fmaxf(-k * ye, dx0), dx1);
+        const float s2 = fmaf(k, ye, x2);
+        const float q = fminf(fmaf(A * s1, s1, D * y1 * y1), fmaf(A * s2, s2, D * ye * ye));
+        return tau > 0.f && !(q > tau);
+    }
+};
 
 __device__ __forceinline__ float warp_sum_f(float v)
 {
@@ -182,7 +187,7 @@ struct SquareGeom {
     int lx, ly;            // tile-local pixel of the lane's pair (left pixel)
     float2 pxc;            // its two pixel-centre x, tile-local
     float pyc;             // its pixel-centre y, tile-local
-    float bx0, bx1, by0, by1; // the square's pixel-centre box, tile-local
+    float bx0, by0;        // the square's first pixel centre, tile-local
 };
 
 template <int TW, int TH> __device__ __forceinline__ SquareGeom square_geom(const CamTable &ct, int tile, int warp,
@@ -200,8 +205,8 @@ template <int TW, int TH> __device__ __forceinline__ SquareGeom square_geom(cons
     q.ly = sy + (lane >> 2);
     q.pxc = make_float2((float)q.lx + 0.5f, (float)q.lx + 1.5f);
     q.pyc = (float)q.ly + 0.5f;
-    q.bx0 = (float)sx + 0.5f; q.bx1 = (float)sx + 7.5f;
-    q.by0 = (float)sy + 0.5f; q.by1 = (float)sy + 7.5f;
+    q.bx0 = (float)sx + 0.5f;
+    q.by0 = (float)sy + 0.5f;
     return q;
 }
 
@@ -236,11 +241,20 @@ __device__ __forceinline__ void put_visits(uint32_t *visits, int start, int b, i
 
 // ---- forward --------------------------------------------------------------
 //
-// Front to back over the visited entries of each batch; a warp stops once all
-// of its pixels have (T would drop below T_min), with no block barrier.  It asks
-// so once per batch: a vote after every entry cost more than the entries it
-// saved (24 mixed views, whole pass: 2.84 ms with it, 2.79 without), as did a
-// vote to skip the entries that reach no live pixel (3.06 ms).
+// The block goes through the tile's list front to back in rounds of 32 entries
+// per warp: each warp stages 32 of them, one per lane, tests each against every
+// square of the tile and leaves a bit mask per square; then every warp walks
+// the round's entries of its own square.  The staged entries are double
+// buffered, so one block barrier per round is enough: a warp that is done
+// with a round stages the next while others still walk.  So every entry is
+// gathered once per tile, and a warp waits for a gather once per round.
+// (Each warp staging every batch for itself, with no barrier, gathered each
+// entry once per warp: 24 mixed views, whole pass, 2.80 ms, this 2.59; the
+// 1080p view of the 5M city 218 and 212 us.)
+// A warp stops walking once all of its pixels have stopped (T would drop below
+// T_min), which it asks once per batch: a vote after every entry cost more than
+// the entries it saved (24 mixed views, whole pass: 2.84 ms with it, 2.79
+// without), as did a vote to skip the entries that reach no live pixel (3.06).
 
 // VISITS: note the entries that composite in each square for the adjoint (not in
 // a forward-only workspace: the bookkeeping costs the walk 6 %).
@@ -254,9 +268,11 @@ __global__ void __launch_bounds__(SquareShape<TW, TH>::threads)
 {
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
     constexpr int kWarps = SquareShape<TW, TH>::warps;
-    __shared__ float4 s0[kWarps][32];
-    __shared__ float4 s1[kWarps][32];
-    __shared__ float s2[kWarps][32];
+    constexpr int kRound = 32 * kWarps; // entries per round
+    __shared__ float4 s0[2][kRound];
+    __shared__ float4 s1[2][kRound];
+    __shared__ float s2[2][kRound];
+    __shared__ unsigned s_mask[2][kWarps][kWarps]; // [square][batch of the round]
     const CamTable &ct = *ctp;
     if ((int)blockIdx.x >= ct.total_tiles) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -268,51 +284,66 @@ __global__ void __launch_bounds__(SquareShape<TW, TH>::threads)
     float2 T = f2(1.f), Cr = f2(0.f), Cg = f2(0.f), Cb = f2(0.f);
     uint32_t last0 = 0, last1 = 0;
     bool dn0 = px >= cam.width || py >= cam.height, dn1 = px + 1 >= cam.width || py >= cam.height;
-    for (int b = start; b < end && !__all_sync(0xffffffffu, dn0 && dn1); b += 32) {
-        const int cnt = min(32, end - b);
-        bool visit = false;
-        if (lane < cnt) {
-            const uint32_t r = vals[b + lane];
-            const float4 r0 = rd0[r], r1 = rd1[r], r2 = rd2[r];
-            const float op = r2.w != 0.f ? 0.f : r1.y; // a record marked culled composites nowhere
-            const float4 e0 = stage_e0_at(r0, r2, q.ox, q.oy);
-            s0[warp][lane] = e0;
-            s1[warp][lane] = make_float4(stage_D(r1), op, r1.z, r1.w);
-            s2[warp][lane] = r2.x;
-            visit = square_visit(r0.z, r0.w, r1.x, op, rc.alpha_min, e0.x, e0.y, q.bx0, q.bx1, q.by0, q.by1);
+    int buf = 0;
+    for (int first = start; first < end; first += kRound, buf ^= 1) {
+        {
+            const int at = 32 * warp + lane;
+            unsigned meets = 0; // squares the entry may composite in
+            if (first + at < end) {
+                const uint32_t r = vals[first + at];
+                const float4 r0 = rd0[r], r1 = rd1[r], r2 = rd2[r];
+                const float op = r2.w != 0.f ? 0.f : r1.y; // a record marked culled composites nowhere
+                const float4 e0 = stage_e0_at(r0, r2, q.ox, q.oy);
+                s0[buf][at] = e0;
+                s1[buf][at] = make_float4(stage_D(r1), op, r1.z, r1.w);
+                s2[buf][at] = r2.x;
+                const SquareTest test(r0, r1.x, op, rc.alpha_min, e0.x, e0.y);
+#pragma unroll
+                for (int k = 0; k < kWarps; k++)
+                    meets |= test.meets(8.f * (k % SquareShape<TW, TH>::wx) + 0.5f, 8.f * (k / SquareShape<TW, TH>::wx) + 0.5f) ? 1u << k : 0u;
+            }
+#pragma unroll
+            for (int k = 0; k < kWarps; k++) {
+                const unsigned m = __ballot_sync(0xffffffffu, (meets >> k) & 1u);
+                if (lane == k) s_mask[buf][k][warp] = m;
+            }
         }
-        unsigned m = __ballot_sync(0xffffffffu, visit);
-        __syncwarp();
-        unsigned comp = 0; // entries that composite in the lane's pixels
-        while (m != 0u) {
-            const int jj = __ffs(m) - 1; // front to back
-            m &= m - 1u;
-            const float4 p0 = s0[warp][jj];
-            const float4 p1 = s1[warp][jj];
-            const uint32_t pos = (uint32_t)(b - start + jj + 1);
-            float2 dx, e;
-            float dy;
-            const float2 pw = pair_power(p0, p1.x, q.pxc, q.pyc, dx, dy, e);
-            float2 G;
-            const float2 al = pair_alpha(pw, p1.y, rc.alpha_max, G);
-            const float2 tT = __ffma2_rn(make_float2(-T.x, -T.y), al, T); // T (1 - alpha)
-            const bool ok0 = !dn0 && al.x >= rc.alpha_min, ok1 = !dn1 && al.y >= rc.alpha_min;
-            const bool st0 = ok0 && tT.x < rc.T_min, st1 = ok1 && tT.y < rc.T_min;
-            const bool c0 = ok0 && !st0, c1 = ok1 && !st1;
-            dn0 = dn0 || st0;
-            dn1 = dn1 || st1;
-            if (VISITS && (c0 || c1)) comp |= 1u << jj;
-            const float2 ae = make_float2(c0 ? al.x : 0.f, c1 ? al.y : 0.f); // skipped fragments add nothing
-            const float2 w = __fmul2_rn(ae, T);
-            Cr = __ffma2_rn(w, f2(p1.z), Cr);
-            Cg = __ffma2_rn(w, f2(p1.w), Cg);
-            Cb = __ffma2_rn(w, f2(s2[warp][jj]), Cb);
-            T = __ffma2_rn(make_float2(-T.x, -T.y), ae, T);
-            last0 = c0 ? pos : last0;
-            last1 = c1 ? pos : last1;
+        if (__syncthreads_and(dn0 && dn1)) break; // the round is staged; every pixel of the tile has stopped
+        for (int sub = 0, b = first; sub < kWarps && b < end; sub++, b += 32) {
+            if (__all_sync(0xffffffffu, dn0 && dn1)) break;
+            unsigned m = s_mask[buf][warp][sub];
+            const float4 *e0s = s0[buf] + 32 * sub, *e1s = s1[buf] + 32 * sub;
+            const float *e2s = s2[buf] + 32 * sub;
+            unsigned comp = 0; // entries that composite in the lane's pixels
+            while (m != 0u) {
+                const int jj = __ffs(m) - 1; // front to back
+                m &= m - 1u;
+                const float4 p0 = e0s[jj];
+                const float4 p1 = e1s[jj];
+                const uint32_t pos = (uint32_t)(b - start + jj + 1);
+                float2 dx, e;
+                float dy;
+                const float2 pw = pair_power(p0, p1.x, q.pxc, q.pyc, dx, dy, e);
+                float2 G;
+                const float2 al = pair_alpha(pw, p1.y, rc.alpha_max, G);
+                const float2 tT = __ffma2_rn(make_float2(-T.x, -T.y), al, T); // T (1 - alpha)
+                const bool ok0 = !dn0 && al.x >= rc.alpha_min, ok1 = !dn1 && al.y >= rc.alpha_min;
+                const bool st0 = ok0 && tT.x < rc.T_min, st1 = ok1 && tT.y < rc.T_min;
+                const bool c0 = ok0 && !st0, c1 = ok1 && !st1;
+                dn0 = dn0 || st0;
+                dn1 = dn1 || st1;
+                if (VISITS && (c0 || c1)) comp |= 1u << jj;
+                const float2 ae = make_float2(c0 ? al.x : 0.f, c1 ? al.y : 0.f); // skipped fragments add nothing
+                const float2 w = __fmul2_rn(ae, T);
+                Cr = __ffma2_rn(w, f2(p1.z), Cr);
+                Cg = __ffma2_rn(w, f2(p1.w), Cg);
+                Cb = __ffma2_rn(w, f2(e2s[jj]), Cb);
+                T = __ffma2_rn(make_float2(-T.x, -T.y), ae, T);
+                last0 = c0 ? pos : last0;
+                last1 = c1 ? pos : last1;
+            }
+            if (VISITS) put_visits<kWarps>(visits, start, b, warp, comp);
         }
-        if (VISITS) put_visits<kWarps>(visits, start, b, warp, comp);
-        __syncwarp();
     }
     const long long np = (long long)cam.width * cam.height;
     float *img = rgb_out + 3 * cam.pix_base;
@@ -694,7 +725,7 @@ __global__ void __launch_bounds__(SquareShape<TW, TH>::threads, SquareShape<TW, 
                 s1[warp][lane] = make_float4(stage_D(r1), r1.y, r2.w != 0.f ? 0.f : r1.y, r2.x);
                 if (FWD) s3[FWD ? warp : 0][lane] = make_float2(r1.z, r1.w);
                 // the record's own opacity: the training opacity is the same or 0
-                visit = square_visit(r0.z, r0.w, r1.x, r1.y, rc.alpha_min, e0.x, e0.y, q.bx0, q.bx1, q.by0, q.by1);
+                visit = SquareTest(r0, r1.x, r1.y, rc.alpha_min, e0.x, e0.y).meets(q.bx0, q.by0);
             }
         }
         const unsigned vmask = __ballot_sync(0xffffffffu, visit);
