@@ -104,8 +104,9 @@ Offsets plan(const gs_capacity &c)
     o.loss_partial_words = fwd_only ? 0 : 2 * 3 * (P / 1024 + 65536);
     o.loss_partial = L.take<float>(o.loss_partial_words);
     // look-back words of the preprocess: two per 128 candidates of the
-    // projection, one per 8192 Gaussians of the gather, and their tickets
-    o.lb_words = 2 * (N / 128) + N / 8192 + 10;
+    // projection, one per block of the gather (640, or one
+    // per 8192 Gaussians), and their tickets
+    o.lb_words = 2 * (N / 128) + N / 8192 + 640 + 10;
     o.lb_status = L.take<unsigned long long>(o.lb_words);
     o.bin_lb_words = T / 1024 + 4; // ... of the binning: 1024 tiles of its scan
     o.bin_lb = L.take<unsigned long long>(o.bin_lb_words);

@@ -595,9 +595,11 @@ __global__ void __launch_bounds__(32 * kGateWarps, 4) gate_count_kernel(GaussPtr
 // takes kGatherChunks chunks: it scans their counts, finds its offset by
 // decoupled look-back (every block publishes after the same little work) and
 // moves its candidates, the loads of four of a thread's in flight together.
-constexpr int kGatherChunks = 64;
-static_assert(kGatherChunks <= 256, "one chunk per thread of the scan");
-template <bool kOneCam>
+// kChunks is 64, or 16 where the blocks then still are few (kGatherFew): a small
+// model's candidates are dense, and 64 chunks of them (8192) keep a block busy
+// for 18 us.  More blocks than that wait on longer look-back chains.
+constexpr int kGatherFew = 640;
+template <bool kOneCam, int kChunks>
 __global__ void __launch_bounds__(256) gate_gather_kernel(PreOut o, const uint16_t *cnt, long long nchunks,
                                                           unsigned long long *lb /* ticket at word 0 */)
 {
@@ -609,8 +611,8 @@ __global__ void __launch_bounds__(256) gate_gather_kernel(PreOut o, const uint16
     if (threadIdx.x == 0) s_bid = atomicAdd((unsigned *)lb, 1u);
     __syncthreads();
     const unsigned bid = s_bid;
-    const long long c0 = (long long)bid * kGatherChunks, c = c0 + threadIdx.x;
-    const unsigned mine = threadIdx.x < kGatherChunks && c < nchunks ? cnt[c] : 0u;
+    const long long c0 = (long long)bid * kChunks, c = c0 + threadIdx.x;
+    const unsigned mine = threadIdx.x < kChunks && c < nchunks ? cnt[c] : 0u;
     unsigned total;
     const unsigned excl = block_exclusive_scan_256<unsigned>(mine, s_warp, total);
     s_incl[threadIdx.x] = excl + mine;
@@ -618,7 +620,7 @@ __global__ void __launch_bounds__(256) gate_gather_kernel(PreOut o, const uint16
         const unsigned long long b = lookback_exclusive(lb + 1, bid, total, o.ctr, kSitePreprocess);
         if (threadIdx.x == 0) {
             s_base = b;
-            if (c0 + kGatherChunks >= nchunks) o.ctr->n_candidates = b + total;
+            if (c0 + kChunks >= nchunks) o.ctr->n_candidates = b + total;
         }
     }
     __syncthreads();
@@ -627,7 +629,7 @@ __global__ void __launch_bounds__(256) gate_gather_kernel(PreOut o, const uint16
     for (unsigned t = threadIdx.x; t < total; t += 256) {
         int lo = 0; // the first chunk whose inclusive count exceeds t
 #pragma unroll
-        for (int step = kGatherChunks / 2; step > 0; step >>= 1) lo += s_incl[lo + step - 1] <= t ? step : 0;
+        for (int step = kChunks / 2; step > 0; step >>= 1) lo += s_incl[lo + step - 1] <= t ? step : 0;
         const long long src = (c0 + lo) * kGateChunk + (t - (lo ? s_incl[lo - 1] : 0u));
         o.cand_g[base + t] = o.gate_g[src];
         if (!kOneCam) o.cand_mask[base + t] = o.gate_mask[src];
@@ -848,8 +850,9 @@ static cudaError_t launch_gate(gs_workspace *ws, cudaStream_t st, const GaussPtr
     launch_pdl(kernel, grid, 32 * kGateWarps, smem, st, gp, o, ws->d_cams, ws->rc, ws->gate_cnt, lb, lb_words, spins);
     kt_end(ws, GS_KT_GATE, st);
     note_launch();
-    launch_pdl(gate_gather_kernel<kOneCam>, (unsigned)((chunks + kGatherChunks - 1) / kGatherChunks), 256, 0, st, o,
-               ws->gate_cnt, chunks, lb);
+    const bool few = (chunks + 15) / 16 <= kGatherFew;
+    launch_pdl(few ? gate_gather_kernel<kOneCam, 16> : gate_gather_kernel<kOneCam, 64>,
+               (unsigned)((chunks + (few ? 15 : 63)) / (few ? 16 : 64)), 256, 0, st, o, ws->gate_cnt, chunks, lb);
     note_launch();
     return cudaGetLastError();
 }
@@ -864,7 +867,7 @@ cudaError_t launch_preprocess(gs_workspace *ws, cudaStream_t st, const uint32_t 
     GaussPtrs gp{ws->g.mean, ws->g.log_scale, ws->g.quat, ws->g.opacity_logit, ws->g.sh, ws->g.lod, n};
     // look-back state (ticket in word 0 of each): the gather's, then the
     // projection's; the gate clears both
-    const long long gather_words = (n + kGateChunk * kGatherChunks - 1) / (kGateChunk * kGatherChunks) + 1;
+    const long long gather_words = std::max<long long>(kGatherFew, n / (64 * kGateChunk) + 1) + 1;
     const long long lb_words = gather_words + 2 * (long long)pchunks + 1;
     if ((size_t)lb_words > ws->lb_words) return cudaErrorInvalidValue; // sized at creation
     PreOut o;
