@@ -188,8 +188,26 @@ def _ptr(t) -> ctypes.c_void_p:
 
 
 def _stream(stream=None) -> ctypes.c_void_p:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return ctypes.c_void_p(stream.cuda_stream)
+    if not torch.cuda.is_initialized():
+        torch.cuda.init()
+    # the current stream's handle alone: torch.cuda.current_stream() builds a Stream object around it,
+    # 4 us for each of a pass's calls
+    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
+
+
+_defaults = None
+
+
+def _default_params() -> "GSRenderParams":
+    """A fresh copy of the library's default parameters (constants, asked for once)."""
+    global _defaults
+    if _defaults is None:
+        p = GSRenderParams()
+        lib().gs_default_params(ctypes.byref(p))
+        _defaults = bytes(p)
+    return GSRenderParams.from_buffer_copy(_defaults)
 
 
 @dataclasses.dataclass
@@ -214,8 +232,7 @@ class RenderParams:
     vis_mass: float | None = None
 
     def c(self) -> GSRenderParams:
-        p = GSRenderParams()
-        lib().gs_default_params(ctypes.byref(p))
+        p = _default_params()
         p.bg = (ctypes.c_float * 3)(*self.bg)
         p.tile_w, p.tile_h = int(self.tile_w), int(self.tile_h)
         p.lod_enable = int(self.lod_enable)
@@ -252,6 +269,10 @@ class GaussianTensors:
     def zeros_like(self) -> "GaussianTensors":
         z = torch.zeros_like
         return GaussianTensors(z(self.mean), z(self.log_scale), z(self.quat), z(self.opacity_logit), z(self.sh), None)
+
+    def empty_like(self) -> "GaussianTensors":
+        e = torch.empty_like
+        return GaussianTensors(e(self.mean), e(self.log_scale), e(self.quat), e(self.opacity_logit), e(self.sh), None)
 
     def params(self):
         return [self.mean, self.log_scale, self.quat, self.opacity_logit, self.sh]
@@ -300,12 +321,15 @@ class ModelTensors:
                        self.v.c_grads() if self.v is not None else none)
 
 
+_F3, _F9 = ctypes.c_float * 3, ctypes.c_float * 9
+
+
 def camera_c(cam) -> GSCamera:
     c = GSCamera()
-    c.R = (ctypes.c_float * 9)(*np.asarray(cam.R, np.float32).ravel())
-    c.t = (ctypes.c_float * 3)(*np.asarray(cam.t, np.float32))
+    c.R = _F9(*np.asarray(cam.R, np.float32).ravel().tolist())
+    c.t = _F3(*np.asarray(cam.t, np.float32).tolist())
     c.fx, c.fy, c.cx, c.cy = float(cam.fx), float(cam.fy), float(cam.cx), float(cam.cy)
-    c.campos = (ctypes.c_float * 3)(*np.asarray(cam.campos, np.float32))
+    c.campos = _F3(*np.asarray(cam.campos, np.float32).tolist())
     c.width, c.height = int(cam.width), int(cam.height)
     return c
 
@@ -642,7 +666,7 @@ class RenderFunction(torch.autograd.Function):
             raise RuntimeError("render backward: the workspace has run another forward since this render's; "
                                "its binning and per-pixel state are gone (use one workspace per pending backward)")
         g = ctx.g
-        grads = g.zeros_like()
+        grads = g.empty_like()  # every row is written
         ctx.ws.render_bwd(g, dL_drgb.contiguous(), grads, accumulate=False)
         return (None, None, None, None, None, grads.mean, grads.log_scale, grads.quat, grads.opacity_logit, grads.sh)
 
