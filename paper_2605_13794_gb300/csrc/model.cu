@@ -156,10 +156,12 @@ __device__ __forceinline__ void write_child(const ScatterArgs &a, long long i, l
     }
 }
 
-// The list of output rows.  Ticket-ordered blocks of 256 Gaussians: each block
-// counts its outputs, finds its offset by decoupled look-back and writes its
-// rows' sources in parent order, with the levels and the split children's mean
-// and scales; model_rows_kernel then copies the rows.
+// The list of output rows.  Ticket-ordered blocks of kListGauss Gaussians (four
+// consecutive ones per thread): each block counts its outputs, finds its offset
+// by decoupled look-back and writes its rows' sources in parent order, with the
+// levels and the split children's mean and scales; model_rows_kernel then
+// copies the rows.
+constexpr int kListItems = 4, kListGauss = 256 * kListItems;
 __global__ void __launch_bounds__(256) model_scatter_kernel(ScatterArgs a)
 {
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
@@ -169,132 +171,135 @@ __global__ void __launch_bounds__(256) model_scatter_kernel(ScatterArgs a)
     if (threadIdx.x == 0) s_bid = atomicAdd((unsigned *)a.lb_status, 1u);
     __syncthreads();
     const unsigned bid = s_bid;
-    const long long i = (long long)bid * 256 + threadIdx.x;
-    int kind = 0;
-    if (i < a.n) kind = a.keep ? (int)((a.keep[i >> 5] >> (i & 31)) & 1u) : densify_kind(a, i);
-    const unsigned long long cnt = kind == 0 ? 0 : (kind == 1 ? 1 : 2);
+    const long long i0 = (long long)bid * kListGauss + threadIdx.x * kListItems;
+    int kind[kListItems];
+    unsigned long long mine = 0;
+    const uint32_t bits = a.keep && i0 < a.n ? a.keep[i0 >> 5] >> (i0 & 31) : 0u;
+#pragma unroll
+    for (int q = 0; q < kListItems; q++) {
+        kind[q] = i0 + q >= a.n ? 0 : a.keep ? (int)((bits >> q) & 1u) : densify_kind(a, i0 + q);
+        mine += kind[q] == 0 ? 0 : (kind[q] == 1 ? 1 : 2);
+    }
     unsigned long long total;
-    const unsigned long long excl = block_exclusive_scan_256<unsigned long long>(cnt, s_warp, total);
+    const unsigned long long excl = block_exclusive_scan_256<unsigned long long>(mine, s_warp, total);
     if (threadIdx.x < 32) {
         const unsigned long long b = lookback_exclusive(a.lb_status + 1, bid, total, a.ctr, kSiteModel);
         if (threadIdx.x == 0) s_base = b;
     }
     __syncthreads();
-    const unsigned long long o = s_base + excl;
-    const unsigned long long nblocks = ((unsigned long long)a.n + 255) / 256;
-    if (bid == nblocks - 1 && threadIdx.x == 0) *a.n_out = (long long)(s_base + total);
-    if (cnt == 0) return;
-    if ((long long)(o + cnt) > a.dst_cap) {
-        set_error(a.ctr, GS_ERR_CAPACITY, kSiteModel);
-        if ((long long)o < a.dst_cap) put_row(a, (long long)o, i, kRowNone); // the first of two rows
-        return;
-    }
-    const long long r = (long long)o;
-    if (kind == 3) {
-        for (int c = 0; c < 2; c++) {
-            put_row(a, r + c, i, kRowChild);
-            write_child(a, i, r + c, c);
+    unsigned long long o = s_base + excl;
+    if (i0 < a.n && i0 + kListItems >= a.n) *a.n_out = (long long)(o + mine); // the last Gaussian's thread
+#pragma unroll
+    for (int q = 0; q < kListItems; q++) {
+        const long long i = i0 + q, r = (long long)o;
+        const unsigned cnt = kind[q] == 0 ? 0 : (kind[q] == 1 ? 1 : 2);
+        o += cnt;
+        if (cnt == 0) continue;
+        if (r + (long long)cnt > a.dst_cap) {
+            set_error(a.ctr, GS_ERR_CAPACITY, kSiteModel);
+            if (r < a.dst_cap) put_row(a, r, i, kRowNone); // the first of two rows
+            continue;
         }
-    } else {
-        put_row(a, r, i, kRowCopy);
-        if (kind == 2) put_row(a, r + 1, i, kRowClone);
-    }
-    if (a.dst.lod) {
-        int lv = a.src.lod ? (int)a.src.lod[i] : 0;
-        if (kind == 3) lv = min(lv + 1, a.max_level); // the next finer level
-        a.dst.lod[r] = (uint8_t)lv;
-        if (cnt == 2) a.dst.lod[r + 1] = (uint8_t)lv;
-    }
-}
-
-// One array of the model, LEN floats per row: output elements in order, four
-// per thread (a float4 where the output is 16-byte aligned, and of one source
-// row where LEN is a multiple of four and the source is aligned too).
-// moment: rows other than plain copies start from zero (all rows without a
-// source array); geom: the split children's values are in place already.  A
-// list entry left unset by a look-back that gave up is not followed (i < n).
-template <int LEN>
-__device__ __forceinline__ void copy_rows(const ScatterArgs &a, const float *__restrict__ src, float *__restrict__ dst,
-                                          long long rows, bool moment, bool geom)
-{
-    if (!dst) return;
-    const bool vdst = ((uintptr_t)dst & 15u) == 0, vsrc = LEN % 4 == 0 && src && ((uintptr_t)src & 15u) == 0;
-    const unsigned long long total = (unsigned long long)rows * LEN, chunks = (total + 3) / 4;
-    const unsigned long long stride = gridDim.x * 256ull;
-#pragma unroll 4 // the loads of four chunks in flight
-    for (unsigned long long c = blockIdx.x * 256ull + threadIdx.x; c < chunks; c += stride) {
-        const unsigned long long e0 = 4 * c;
-        float v[4] = {0.f, 0.f, 0.f, 0.f};
-        bool put = true; // all four elements are written
-        if (LEN % 4 == 0) {
-            const long long o = (long long)(e0 / LEN);
-            const int how = a.how[o];
-            const long long i = (o < a.list_n ? a.list0 : a.list1 - a.list_n)[o];
-            put = i < a.n && how != kRowNone && !(geom && how == kRowChild);
-            if (put && src && !(moment && how != kRowCopy)) {
-                const float *s = src + i * LEN + (long long)(e0 % LEN);
-                if (vsrc) {
-                    const float4 q = __ldcs(reinterpret_cast<const float4 *>(s));
-                    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
-                } else {
-#pragma unroll
-                    for (int u = 0; u < 4; u++) v[u] = s[u];
-                }
-            }
-            if (!put) continue;
-            if (vdst) __stcs(reinterpret_cast<float4 *>(dst + e0), make_float4(v[0], v[1], v[2], v[3]));
-            else {
-#pragma unroll
-                for (int u = 0; u < 4; u++) dst[e0 + u] = v[u];
+        if (kind[q] == 3) {
+            for (int c = 0; c < 2; c++) {
+                put_row(a, r + c, i, kRowChild);
+                write_child(a, i, r + c, c);
             }
         } else {
-            bool w[4];
+            put_row(a, r, i, kRowCopy);
+            if (kind[q] == 2) put_row(a, r + 1, i, kRowClone);
+        }
+        if (a.dst.lod) {
+            int lv = a.src.lod ? (int)a.src.lod[i] : 0;
+            if (kind[q] == 3) lv = min(lv + 1, a.max_level); // the next finer level
+            a.dst.lod[r] = (uint8_t)lv;
+            if (cnt == 2) a.dst.lod[r + 1] = (uint8_t)lv;
+        }
+    }
+}
+
+// A warp's 32 output rows of one array, LEN floats each, from row base on; lane
+// r holds row r's source Gaussian i.  Consecutive lanes move consecutive
+// elements (float4 where the rows are whole float4s of aligned arrays), up to
+// four loads of a lane in flight.  Rows of `write` are written, those of `read`
+// with the source's values, the others (and all without a source array) with
+// zeros.
+template <int LEN, bool VEC>
+__device__ __forceinline__ void copy_rows(const float *__restrict__ src, float *__restrict__ dst, long long base,
+                                          uint32_t i, unsigned write, unsigned read)
+{
+    if (!dst) return;
+    constexpr int W = VEC && LEN % 4 == 0 ? 4 : 1, kPer = LEN / W; // elements moved at once, moves per row
+    constexpr int kIn = kPer < 4 ? kPer : 4;                       // loads in flight
+    static_assert(kPer % kIn == 0, "whole groups of loads");
+    const int lane = threadIdx.x & 31;
+    if (!src) read = 0u;
+#pragma unroll 1
+    for (int g = 0; g < kPer; g += kIn) {
+        float4 v[kIn];
 #pragma unroll
-            for (int u = 0; u < 4; u++) {
-                const unsigned long long e = e0 + u;
-                w[u] = e < total;
-                if (w[u]) {
-                    const long long o = (long long)(e / LEN);
-                    const int how = a.how[o];
-                    const long long i = (o < a.list_n ? a.list0 : a.list1 - a.list_n)[o];
-                    w[u] = i < a.n && how != kRowNone && !(geom && how == kRowChild);
-                    if (w[u] && src && !(moment && how != kRowCopy)) v[u] = src[i * LEN + (long long)(e % LEN)];
-                }
-                put = put && w[u];
+        for (int q = 0; q < kIn; q++) {
+            const int e = (g + q) * 32 + lane, row = e / kPer;
+            const size_t from = (size_t)__shfl_sync(0xffffffffu, i, row) * LEN + (e % kPer) * W;
+            v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if ((read >> row) & 1u) {
+                if (W == 4) v[q] = __ldcs(reinterpret_cast<const float4 *>(src + from));
+                else v[q].x = __ldcs(src + from);
             }
-            if (put && vdst) __stcs(reinterpret_cast<float4 *>(dst + e0), make_float4(v[0], v[1], v[2], v[3]));
-            else {
+        }
 #pragma unroll
-                for (int u = 0; u < 4; u++)
-                    if (w[u]) dst[e0 + u] = v[u];
+        for (int q = 0; q < kIn; q++) {
+            const int e = (g + q) * 32 + lane, row = e / kPer;
+            if ((write >> row) & 1u) {
+                float *to = dst + (size_t)base * LEN + (size_t)e * W;
+                if (W == 4) __stcs(reinterpret_cast<float4 *>(to), v[q]);
+                else __stcs(to, v[q].x);
             }
         }
     }
 }
 
-// The rows of the list, array by array: consecutive threads write consecutive
-// output elements and read consecutive elements of a source row, so both
-// sides move whole sectors.  Bound by HBM (708 bytes read and written per row
-// of a model with moments).
-__global__ void __launch_bounds__(256, 4) model_rows_kernel(ScatterArgs a)
+// The rows of the list, 32 per warp, array by array.  Bound by HBM (708 bytes
+// read and written per row of a model with moments).  One thread per Gaussian
+// copying its 177 floats one after another, as the list kernel once did, touched
+// a sector per float: the mass cut and compaction of 3M Gaussians with moments
+// took 2.52 ms and takes 0.98, the density control of 1.5M 2.32 and 0.67 (array by
+// array over the whole model, 62 registers: 1.14 and 0.82).  (A list entry left unset by a look-back that gave up is
+// not followed: i < n.)
+template <bool VEC> __global__ void __launch_bounds__(256, 8) model_rows_kernel(ScatterArgs a)
 {
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
     const long long rows = min(*a.n_out, a.dst_cap);
-    copy_rows<48>(a, a.src.p[4], a.dst.p[4], rows, false, false);
-    copy_rows<48>(a, a.src.m[4], a.dst.m[4], rows, true, false);
-    copy_rows<48>(a, a.src.v[4], a.dst.v[4], rows, true, false);
-    copy_rows<4>(a, a.src.p[2], a.dst.p[2], rows, false, false);
-    copy_rows<4>(a, a.src.m[2], a.dst.m[2], rows, true, false);
-    copy_rows<4>(a, a.src.v[2], a.dst.v[2], rows, true, false);
-#pragma unroll 1
-    for (int k = 0; k < 2; k++) { // mean, log-scale
-        copy_rows<3>(a, a.src.p[k], a.dst.p[k], rows, false, true);
-        copy_rows<3>(a, a.src.m[k], a.dst.m[k], rows, true, false);
-        copy_rows<3>(a, a.src.v[k], a.dst.v[k], rows, true, false);
+    const int lane = threadIdx.x & 31;
+    for (long long base = ((long long)blockIdx.x * 8 + (threadIdx.x >> 5)) * 32; base < rows;
+         base += (long long)gridDim.x * 256) {
+        const long long o = base + lane;
+        uint32_t i = 0;
+        int how = kRowNone;
+        if (o < rows) {
+            i = (o < a.list_n ? a.list0 : a.list1 - a.list_n)[o];
+            how = (long long)i < a.n ? a.how[o] : kRowNone;
+            if (how == kRowNone) i = 0;
+        }
+        const unsigned put = __ballot_sync(0xffffffffu, how != kRowNone);
+        const unsigned whole = __ballot_sync(0xffffffffu, how == kRowCopy); // rows that keep their moments
+        const unsigned geom = __ballot_sync(0xffffffffu, how != kRowNone && how != kRowChild);
+        copy_rows<48, VEC>(a.src.p[4], a.dst.p[4], base, i, put, put);
+        copy_rows<48, VEC>(a.src.m[4], a.dst.m[4], base, i, put, whole);
+        copy_rows<48, VEC>(a.src.v[4], a.dst.v[4], base, i, put, whole);
+        copy_rows<4, VEC>(a.src.p[2], a.dst.p[2], base, i, put, put);
+        copy_rows<4, VEC>(a.src.m[2], a.dst.m[2], base, i, put, whole);
+        copy_rows<4, VEC>(a.src.v[2], a.dst.v[2], base, i, put, whole);
+#pragma unroll
+        for (int k = 0; k < 2; k++) { // mean, log-scale: a split child's are in place already
+            copy_rows<3, VEC>(a.src.p[k], a.dst.p[k], base, i, geom, geom);
+            copy_rows<3, VEC>(a.src.m[k], a.dst.m[k], base, i, put, whole);
+            copy_rows<3, VEC>(a.src.v[k], a.dst.v[k], base, i, put, whole);
+        }
+        copy_rows<1, VEC>(a.src.p[3], a.dst.p[3], base, i, put, put);
+        copy_rows<1, VEC>(a.src.m[3], a.dst.m[3], base, i, put, whole);
+        copy_rows<1, VEC>(a.src.v[3], a.dst.v[3], base, i, put, whole);
     }
-    copy_rows<1>(a, a.src.p[3], a.dst.p[3], rows, false, false);
-    copy_rows<1>(a, a.src.m[3], a.dst.m[3], rows, true, false);
-    copy_rows<1>(a, a.src.v[3], a.dst.v[3], rows, true, false);
 }
 
 // Views in which each Gaussian has a record (+= per Gaussian; records of a
@@ -358,7 +363,7 @@ cudaError_t launch_prune_mass(gs_workspace *ws, cudaStream_t st, const float *s,
 
 cudaError_t launch_model_scatter(gs_workspace *ws, cudaStream_t st, ScatterArgs &a)
 {
-    const unsigned long long blocks = ((unsigned long long)a.n + 255) / 256;
+    const unsigned long long blocks = ((unsigned long long)a.n + kListGauss - 1) / kListGauss;
     cudaError_t e;
     if ((e = cudaMemsetAsync(ws->mlb, 0, (blocks + 1) * sizeof(unsigned long long), st)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(a.n_out, 0, sizeof(long long), st)) != cudaSuccess) return e;
@@ -373,7 +378,12 @@ cudaError_t launch_model_scatter(gs_workspace *ws, cudaStream_t st, ScatterArgs 
     a.how = reinterpret_cast<uint8_t *>(ws->mval[0]);
     launch_pdl(model_scatter_kernel, (unsigned)blocks, 256, 0, st, a);
     note_launch();
-    launch_pdl(model_rows_kernel, 8u * (unsigned)ws->sm_count, 256, 0, st, a);
+    // the SH and quaternion rows move as float4 where every such array is 16-byte aligned
+    bool vec = true;
+    for (const ModelRows *r : {&a.src, &a.dst})
+        for (int k : {2, 4})
+            for (const float *p : {r->p[k], r->m[k], r->v[k]}) vec = vec && ((uintptr_t)p & 15u) == 0;
+    launch_pdl(vec ? model_rows_kernel<true> : model_rows_kernel<false>, 8u * (unsigned)ws->sm_count, 256, 0, st, a);
     note_launch();
     return cudaGetLastError();
 }
