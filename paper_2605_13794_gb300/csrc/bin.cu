@@ -36,7 +36,7 @@ constexpr int kBinThreads = 128;       // threads per block of the count and sca
 constexpr int kBinItems = kBinChunk / kBinThreads; // instances per thread
 constexpr int kTileScanItems = 4;      // tiles per thread of the tile scan (1024 per block)
 constexpr int kSortWarps = 4;          // warps (and tiles) per block of the per-tile sort
-constexpr int kWarpSort = 128;         // entries one warp sorts alone (4 per lane)
+constexpr int kWarpSort = 256;         // entries one warp sorts alone (8 per lane)
 constexpr int kBlockSort = 2048;       // entries a block sorts in shared memory (16 per lane)
 
 struct BinArgs {
@@ -277,25 +277,111 @@ __device__ __forceinline__ uint32_t merge_split(const uint2 *x, uint32_t nx, con
     return lo;
 }
 
-// The n <= 32 * E keys at p in the warp's registers, padded with the largest
-// key (in any order: consecutive lanes read consecutive keys).
-template <int E> __device__ __forceinline__ void load_keys(const uint2 *p, uint32_t n, unsigned long long (&x)[E])
+// The same network on 32-bit keys: a shuffle and a minimum or maximum per element
+// and stage, against two shuffles, a 64-bit compare and two selects.  Within runs
+// shorter than E the direction is the register's, known to the compiler, and from
+// there on the lane's alone, one flag per stage (computed per element, as above,
+// it cost as much as the exchange: 28 us for 24 in the 5M city at 1080p).
+template <int E> __device__ __forceinline__ void warp_sort_regs(unsigned (&x)[E])
 {
     const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int e = 0; e < E; e++) x[e] = (uint32_t)(e * 32 + lane) < n ? key_of(p[e * 32 + lane]) : ~0ull;
+    for (int size = 2; size < E; size <<= 1) {
+#pragma unroll
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+#pragma unroll
+            for (int e = 0; e < E; e++) {
+                if (e & stride) continue; // the lower element of each pair
+                const unsigned u = x[e], v = x[e ^ stride];
+                x[e] = e & size ? max(u, v) : min(u, v);
+                x[e ^ stride] = e & size ? min(u, v) : max(u, v);
+            }
+        }
+    }
+    for (int run = E > 1 ? 1 : 2; run <= 32; run <<= 1) { // runs of E * run elements
+        const bool up = (lane & run) == 0;
+        for (int ls = run >> 1; ls > 0; ls >>= 1) {
+            const bool least = ((lane & ls) == 0) == up;
+#pragma unroll
+            for (int e = 0; e < E; e++) {
+                const unsigned v = __shfl_xor_sync(0xffffffffu, x[e], ls);
+                x[e] = least ? min(x[e], v) : max(x[e], v);
+            }
+        }
+#pragma unroll
+        for (int stride = E / 2; stride > 0; stride >>= 1) {
+#pragma unroll
+            for (int e = 0; e < E; e++) {
+                if (e & stride) continue;
+                const unsigned u = x[e], v = x[e ^ stride];
+                x[e] = up ? min(u, v) : max(u, v);
+                x[e ^ stride] = up ? max(u, v) : min(u, v);
+            }
+        }
+    }
+}
+
+// The warp's n <= 32 * E keys at p in order: y[e] of lane l is key E l + e, the
+// places past n hold the largest key.  The keys are ordered by 32 bits, the
+// depth above the list's least one in as many bits as the place in the list
+// leaves (all of them in a list whose depths lie within one binade or so) and
+// that place, which fetches the key from its copy in shared memory (stage, 32 E
+// of the warp's own).  Two keys that agree in those depth bits (equal depths,
+// above all) are in no order: then the 64-bit network sorts the list.
+// kWarpSort is 256: with 128, the lists of 129 to 256 entries go to the block and
+// the importance pass of eight views takes 1018 us for 1015.
+template <int E>
+__device__ __forceinline__ void sort_keys(const uint2 *p, uint32_t n, unsigned long long *stage,
+                                          unsigned long long (&y)[E])
+{
+    constexpr int kBits = E == 1 ? 5 : E == 2 ? 6 : E == 4 ? 7 : E == 8 ? 8 : 9; // log2(32 E)
+    const int lane = threadIdx.x & 31;
+    unsigned x[E], least = ~0u, most = 0u;
+#pragma unroll
+    for (int e = 0; e < E; e++) {
+        const uint32_t g = (uint32_t)(e * 32 + lane);
+        const uint2 q = g < n ? p[g] : make_uint2(~0u, ~0u);
+        stage[g] = key_of(q);
+        x[e] = q.x;
+        least = min(least, q.x);
+        most = max(most, g < n ? q.x : 0u);
+    }
+    least = __reduce_min_sync(0xffffffffu, least);
+    most = __reduce_max_sync(0xffffffffu, most);
+    const int shift = max(0, 32 - __clz(most - least) + kBits - 32);
+#pragma unroll
+    for (int e = 0; e < E; e++) {
+        const uint32_t g = (uint32_t)(e * 32 + lane);
+        x[e] = g < n ? ((x[e] - least) >> shift) << kBits | g : ~0u;
+    }
+    warp_sort_regs<E>(x);
+    __syncwarp(); // the staged keys are in place
+    bool clash = false;
+    const unsigned next = __shfl_down_sync(0xffffffffu, x[0], 1);
+#pragma unroll
+    for (int e = 0; e < E; e++) {
+        const unsigned after = e + 1 < E ? x[e + 1 < E ? e + 1 : 0] : next;
+        clash = clash || ((x[e] ^ after) >> kBits == 0u && (uint32_t)(lane * E + e + 1) < n);
+        y[e] = stage[x[e] & (32u * E - 1u)];
+    }
+    if (__any_sync(0xffffffffu, clash)) {
+#pragma unroll
+        for (int e = 0; e < E; e++) y[e] = stage[e * 32 + lane];
+        warp_sort_regs<E>(y);
+    }
+    __syncwarp(); // the staged keys are read
 }
 
 // One warp sorts the n <= 32 * E keys at p and writes the records in order.
-template <int E> __device__ __forceinline__ void warp_sort(const uint2 *p, uint32_t n, uint32_t *out)
+template <int E>
+__device__ __forceinline__ void warp_sort(const uint2 *p, uint32_t n, unsigned long long *stage, uint32_t *out)
 {
     const int lane = threadIdx.x & 31;
-    unsigned long long x[E];
-    load_keys<E>(p, n, x);
-    warp_sort_regs<E>(x);
+    unsigned long long y[E];
+    sort_keys<E>(p, n, stage, y);
 #pragma unroll
     for (int e = 0; e < E; e++)
-        if ((uint32_t)(lane * E + e) < n) out[lane * E + e] = (uint32_t)x[e];
+        if ((uint32_t)(lane * E + e) < n) out[lane * E + e] = (uint32_t)y[e];
 }
 
 // The block sorts the n <= 32 * E * kSortWarps keys at p: each warp a run of a
@@ -310,11 +396,10 @@ __device__ __forceinline__ void block_sort(const uint2 *p, uint32_t n, unsigned 
     const uint32_t run = (n + kSortWarps - 1) / kSortWarps;
     const uint32_t first = min(warp * run, n), len = min(run, n - first);
     {
-        unsigned long long x[E];
-        load_keys<E>(p + first, len, x);
-        warp_sort_regs<E>(x);
+        unsigned long long y[E];
+        sort_keys<E>(p + first, len, s[warp], y);
 #pragma unroll
-        for (int e = 0; e < E; e++) s[warp][lane * E + e] = x[e];
+        for (int e = 0; e < E; e++) s[warp][lane * E + e] = y[e];
     }
     __syncthreads();
     for (uint32_t i = lane; i < len; i += 32) {
@@ -371,9 +456,11 @@ __global__ void __launch_bounds__(32 * kSortWarps, 8) tile_sort_kernel(BinArgs a
     if (mine > 0 && mine <= (uint32_t)kWarpSort) {
         const uint2 *p = a.pairs + rg.x;
         uint32_t *out = a.sval + rg.x;
-        if (mine <= 32) warp_sort<1>(p, mine, out);
-        else if (mine <= 64) warp_sort<2>(p, mine, out);
-        else warp_sort<4>(p, mine, out);
+        unsigned long long *stage = s_run[warp];
+        if (mine <= 32) warp_sort<1>(p, mine, stage, out);
+        else if (mine <= 64) warp_sort<2>(p, mine, stage, out);
+        else if (mine <= 128) warp_sort<4>(p, mine, stage, out);
+        else warp_sort<8>(p, mine, stage, out);
     }
     if (!__syncthreads_or(mine > (uint32_t)kWarpSort)) return;
     for (int w = 0; w < kSortWarps; w++) {

@@ -88,3 +88,27 @@ def test_too_few_instances_is_reported_and_the_next_binning_is_whole():
     ws.sync_status()
     _check(ws, cam, 2500)
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("depths", ["near", "wide", "pairs", "equal"])
+@pytest.mark.parametrize("n", [2, 31, 33, 64, 127, 128, 129, 255, 256, 257, 511, 1025, 2048, 4100])
+def test_depths_that_fit_a_sort_word_and_those_that_do_not(n, depths):
+    """Distinct depths in one binade (their bits fit beside the place), over eight
+    decades (cut bits: distinct or clashing), a single equal pair, all equal."""
+    cam = synth.plain_camera(16, 16, 20.0)
+    g = synth.plain_scene(n, seed=n)
+    rng = np.random.default_rng(n)
+    z = 4.0 + rng.permutation(n).astype(np.float32) * np.float32(3.0 / n)
+    if depths == "wide":
+        z = 10.0 ** rng.uniform(0.0, 8.0, n)
+    elif depths == "pairs":
+        z[-1] = z[0]
+    elif depths == "equal":
+        z[:] = 5.0
+    g.mean[:, :2] = 0.0
+    g.mean[:, 2] = z
+    ws = B.Workspace(max_gaussians=n, max_records=n, max_instances=n, max_tiles=1, max_pixels=256)
+    ws.preprocess(B.GaussianTensors.from_host(g), [cam], B.RenderParams())
+    ws.bin_sort()
+    ws.sync_status()
+    assert _check(ws, cam, n) == n
