@@ -14,9 +14,18 @@
 
 namespace gs {
 
-constexpr int kLT = 32;           // output tile edge
+constexpr int kLT = 32;           // output tile edge (width, in the forward)
 constexpr int kHalo = 5;          // window radius
 constexpr int kLTH = kLT + 2 * kHalo;
+// The forward's tile is 36 rows by six warps: its 46 rows with the halo by four
+// segments of eight are 184 of 192 threads of the horizontal pass (of 32 rows, 168
+// of 256), and six rows a thread of the vertical pass read 16 values instead of
+// 14 for four.  Both passes are bound by issue slots and the latency between the
+// barriers: two 1201 x 1599 views took 108 us and take 98, eight of 1600 x 1200
+// 410 and 367.  (42 rows by seven warps: 103; 48 by eight: 105; 30 by five: 100.
+// The adjoint, of fewer maps, is no faster in either form: 88 us.)
+constexpr int kFwdRows = 36, kFwdWarps = 6, kFwdThreads = 32 * kFwdWarps;
+constexpr int kFwdRowsH = kFwdRows + 2 * kHalo;
 
 struct Win {
     float w[6]; // taps 0 .. 5; tap t > 5 is tap 10 - t
@@ -36,10 +45,13 @@ __device__ __forceinline__ float ld_zero(const float *p, int H, int W, int y, in
 // advances two maps.
 constexpr int kHSeg = 8;                 // horizontal outputs per thread (42 rows x 4 segments)
 constexpr int kVSeg = 4;                 // vertical outputs per thread (32 columns x 8 segments)
+constexpr int kFwdVSeg = kFwdRows / kFwdWarps; // and the forward's
 constexpr int kLTP = kLTH + 1;           // padded row of the staged tile
 // staging: warp w loads rows w, w + 8, ... of the tile with its halo, lane l
 // columns l and l + 32
 constexpr int kStageRows = (kLTH + 7) / 8;
+constexpr int kFwdStageRows = (kFwdRowsH + kFwdWarps - 1) / kFwdWarps;
+static_assert(kFwdVSeg * kFwdWarps == kFwdRows, "whole segments");
 static_assert(kLTH <= 64, "two columns per lane cover a staged row");
 
 __device__ __forceinline__ float2 f2s(float a) { return make_float2(a, a); }
@@ -60,48 +72,48 @@ __device__ __forceinline__ void window_pairs(const Win &win, float2 (&w)[6])
 
 // grid: (tiles_x, tiles_y, batch * 3).  F: the three coefficient maps of the
 // SSIM gradient of each plane, planar: F[(plane * 3 + m) * H * W + pixel].
-__global__ void __launch_bounds__(256, 4) ssim_fwd_kernel(const float *img, const float *tgt, int H, int W, Win win,
+__global__ void __launch_bounds__(kFwdThreads, 4) ssim_fwd_kernel(const float *img, const float *tgt, int H, int W, Win win,
                                                        float C1, float C2, float *F, unsigned long long *acc)
 {
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
-    __shared__ float2 sxy[kLTH][kLTP];
-    __shared__ float2 hb01[kLTH][kLT + 1], hb23[kLTH][kLT + 1];
-    __shared__ float hb4[kLTH][kLT + 1];
-    __shared__ float red[2][8];
+    __shared__ float2 sxy[kFwdRowsH][kLTP];
+    __shared__ float2 hb01[kFwdRowsH][kLT + 1], hb23[kFwdRowsH][kLT + 1];
+    __shared__ float hb4[kFwdRowsH][kLT + 1];
+    __shared__ float red[2][kFwdWarps];
     const int plane = blockIdx.z;
     float2 w[6];
     window_pairs(win, w);
     const float *x = img + (long long)plane * H * W;
     const float *y = tgt + (long long)plane * H * W;
-    const int ox = blockIdx.x * kLT, oy = blockIdx.y * kLT;
+    const int ox = blockIdx.x * kLT, oy = blockIdx.y * kFwdRows;
     {
         // every load of the thread issued before the first store
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        float2 buf[kStageRows][2];
+        float2 buf[kFwdStageRows][2];
 #pragma unroll
-        for (int q = 0; q < kStageRows; q++)
+        for (int q = 0; q < kFwdStageRows; q++)
 #pragma unroll
             for (int h = 0; h < 2; h++) {
-                const int r = warp + 8 * q, c = lane + 32 * h;
+                const int r = warp + kFwdWarps * q, c = lane + 32 * h;
                 const int gy = oy + r - kHalo, gx = ox + c - kHalo;
-                buf[q][h] = r < kLTH && c < kLTH ? make_float2(ld_zero(x, H, W, gy, gx), ld_zero(y, H, W, gy, gx))
+                buf[q][h] = r < kFwdRowsH && c < kLTH ? make_float2(ld_zero(x, H, W, gy, gx), ld_zero(y, H, W, gy, gx))
                                                  : make_float2(0.f, 0.f);
             }
 #pragma unroll
-        for (int q = 0; q < kStageRows; q++)
+        for (int q = 0; q < kFwdStageRows; q++)
 #pragma unroll
             for (int h = 0; h < 2; h++) {
-                const int r = warp + 8 * q, c = lane + 32 * h;
-                if (r < kLTH && c < kLTH) sxy[r][c] = buf[q][h];
+                const int r = warp + kFwdWarps * q, c = lane + 32 * h;
+                if (r < kFwdRowsH && c < kLTH) sxy[r][c] = buf[q][h];
             }
     }
     __syncthreads();
-    // horizontal blur of (x, y), (x^2, y^2) and xy: 42 rows x (32 / kHSeg) segments,
+    // horizontal blur of (x, y), (x^2, y^2) and xy: 46 rows x (32 / kHSeg) segments,
     // consecutive threads on consecutive rows (no bank conflicts)
     // input by input: each input's products x^2, y^2 and xy are formed once and
     // added to the kHSeg outputs whose window holds it
-    for (int wi = threadIdx.x; wi < kLTH * (kLT / kHSeg); wi += 256) {
-        const int r = wi % kLTH, c0 = (wi / kLTH) * kHSeg;
+    for (int wi = threadIdx.x; wi < kFwdRowsH * (kLT / kHSeg); wi += kFwdThreads) {
+        const int r = wi % kFwdRowsH, c0 = (wi / kFwdRowsH) * kHSeg;
         float2 a01[kHSeg], a23[kHSeg];
         float a4[kHSeg];
 #pragma unroll
@@ -126,20 +138,20 @@ __global__ void __launch_bounds__(256, 4) ssim_fwd_kernel(const float *img, cons
         for (int o = 0; o < kHSeg; o++) { hb01[r][c0 + o] = a01[o]; hb23[r][c0 + o] = a23[o]; hb4[r][c0 + o] = a4[o]; }
     }
     __syncthreads();
-    // vertical blur and the SSIM terms: 32 columns x (32 / kVSeg) segments
+    // vertical blur and the SSIM terms: 32 columns x kFwdWarps segments
     float ssum = 0.f, l1sum = 0.f;
     {
-        const int c = threadIdx.x % kLT, r0 = (threadIdx.x / kLT) * kVSeg;
-        float2 m01[kVSeg], m23[kVSeg];
-        float m4[kVSeg];
+        const int c = threadIdx.x % kLT, r0 = (threadIdx.x / kLT) * kFwdVSeg;
+        float2 m01[kFwdVSeg], m23[kFwdVSeg];
+        float m4[kFwdVSeg];
 #pragma unroll
-        for (int o = 0; o < kVSeg; o++) { m01[o] = f2s(0.f); m23[o] = f2s(0.f); m4[o] = 0.f; }
+        for (int o = 0; o < kFwdVSeg; o++) { m01[o] = f2s(0.f); m23[o] = f2s(0.f); m4[o] = 0.f; }
 #pragma unroll
-        for (int j = 0; j < kVSeg + 10; j++) {
+        for (int j = 0; j < kFwdVSeg + 10; j++) {
             const float2 v01 = hb01[r0 + j][c], v23 = hb23[r0 + j][c];
             const float v4 = hb4[r0 + j][c];
 #pragma unroll
-            for (int o = 0; o < kVSeg; o++) {
+            for (int o = 0; o < kFwdVSeg; o++) {
                 const int t = j - o;
                 if (t >= 0 && t < 11) {
                     const float2 wt = w[tap(t)];
@@ -150,7 +162,7 @@ __global__ void __launch_bounds__(256, 4) ssim_fwd_kernel(const float *img, cons
             }
         }
 #pragma unroll
-        for (int o = 0; o < kVSeg; o++) {
+        for (int o = 0; o < kFwdVSeg; o++) {
             const int r = r0 + o;
             const int gy = oy + r, gx = ox + c;
             if (gy >= H || gx >= W) continue;
@@ -181,7 +193,7 @@ __global__ void __launch_bounds__(256, 4) ssim_fwd_kernel(const float *img, cons
     __syncthreads();
     if (threadIdx.x == 0) {
         float a = 0.f, b = 0.f;
-        for (int q = 0; q < 8; q++) { a += red[0][q]; b += red[1][q]; }
+        for (int q = 0; q < kFwdWarps; q++) { a += red[0][q]; b += red[1][q]; }
         // the view's sums in 64-bit fixed point (24 fractional bits): integer
         // atomics add exactly, so the totals do not depend on block order
         const int view = blockIdx.z / 3;
@@ -319,12 +331,13 @@ cudaError_t launch_loss(gs_workspace *ws, cudaStream_t st, const float *img, con
     for (int k = 0; k < 11; k++) { g[k] = exp(-((k - 5) * (k - 5)) / (2.0 * 1.5 * 1.5)); sum += g[k]; }
     for (int k = 0; k < 6; k++) win.w[k] = (float)(g[k] / sum);
     const dim3 grid((W + kLT - 1) / kLT, (H + kLT - 1) / kLT, B * 3);
+    const dim3 fgrid(grid.x, (H + kFwdRows - 1) / kFwdRows, B * 3);
     float *maps = ws->loss_maps; // three planes per image plane
     unsigned long long *acc = reinterpret_cast<unsigned long long *>(ws->loss_partial); // [B][2]
     cudaError_t e = cudaMemsetAsync(acc, 0, 2 * (size_t)B * sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
     kt_begin(ws, GS_KT_SSIM_FWD, st);
-    launch_pdl(ssim_fwd_kernel, grid, 256, 0, st, img, tgt, H, W, win, 0.01f * 0.01f, 0.03f * 0.03f, maps, acc);
+    launch_pdl(ssim_fwd_kernel, fgrid, kFwdThreads, 0, st, img, tgt, H, W, win, 0.01f * 0.01f, 0.03f * 0.03f, maps, acc);
     kt_end(ws, GS_KT_SSIM_FWD, st);
     note_launch();
     kt_begin(ws, GS_KT_SSIM_BWD, st);
