@@ -17,15 +17,18 @@ namespace gs {
 constexpr int kLT = 32;           // output tile edge (width, in the forward)
 constexpr int kHalo = 5;          // window radius
 constexpr int kLTH = kLT + 2 * kHalo;
-// The forward's tile is 36 rows by six warps: its 46 rows with the halo by four
-// segments of eight are 184 of 192 threads of the horizontal pass (of 32 rows, 168
-// of 256), and six rows a thread of the vertical pass read 16 values instead of
-// 14 for four.  Both passes are bound by issue slots and the latency between the
-// barriers: two 1201 x 1599 views took 108 us and take 98, eight of 1600 x 1200
-// 410 and 367.  (42 rows by seven warps: 103; 48 by eight: 105; 30 by five: 100.
-// The adjoint, of fewer maps, is no faster in either form: 88 us.)
-constexpr int kFwdRows = 36, kFwdWarps = 6, kFwdThreads = 32 * kFwdWarps;
-constexpr int kFwdRowsH = kFwdRows + 2 * kHalo;
+// The forward's tile has WARPS x SEG rows, a warp SEG of them in the vertical pass.
+// Both passes are bound by issue slots and the latency between the barriers.  36 rows
+// by six warps: the 46 rows with the halo by four segments of eight are 184 of 192
+// threads of the horizontal pass (32 rows by eight: 168 of 256), and six rows a thread
+// of the vertical pass read 16 values instead of 14 for four.  Two 1201 x 1599 views
+// took 108 us and take 98, eight of 1600 x 1200 410 and 367.  (42 rows by seven warps:
+// 103; 48 by eight: 105; 30 by five: 100.  The adjoint, of fewer maps, is no faster in
+// either form: 88 us.)
+template <int WARPS, int SEG> struct FwdTile {
+    static constexpr int threads = 32 * WARPS, rows = WARPS * SEG, rows_h = rows + 2 * kHalo;
+    static constexpr int stage_rows = (rows_h + WARPS - 1) / WARPS; // rows a warp stages
+};
 
 struct Win {
     float w[6]; // taps 0 .. 5; tap t > 5 is tap 10 - t
@@ -45,13 +48,10 @@ __device__ __forceinline__ float ld_zero(const float *p, int H, int W, int y, in
 // advances two maps.
 constexpr int kHSeg = 8;                 // horizontal outputs per thread (42 rows x 4 segments)
 constexpr int kVSeg = 4;                 // vertical outputs per thread (32 columns x 8 segments)
-constexpr int kFwdVSeg = kFwdRows / kFwdWarps; // and the forward's
 constexpr int kLTP = kLTH + 1;           // padded row of the staged tile
 // staging: warp w loads rows w, w + 8, ... of the tile with its halo, lane l
 // columns l and l + 32
 constexpr int kStageRows = (kLTH + 7) / 8;
-constexpr int kFwdStageRows = (kFwdRowsH + kFwdWarps - 1) / kFwdWarps;
-static_assert(kFwdVSeg * kFwdWarps == kFwdRows, "whole segments");
 static_assert(kLTH <= 64, "two columns per lane cover a staged row");
 
 __device__ __forceinline__ float2 f2s(float a) { return make_float2(a, a); }
@@ -72,48 +72,50 @@ __device__ __forceinline__ void window_pairs(const Win &win, float2 (&w)[6])
 
 // grid: (tiles_x, tiles_y, batch * 3).  F: the three coefficient maps of the
 // SSIM gradient of each plane, planar: F[(plane * 3 + m) * H * W + pixel].
-__global__ void __launch_bounds__(kFwdThreads, 4) ssim_fwd_kernel(const float *img, const float *tgt, int H, int W, Win win,
-                                                       float C1, float C2, float *F, unsigned long long *acc)
+template <int WARPS, int SEG>
+__global__ void __launch_bounds__(32 * WARPS, 4) ssim_fwd_kernel(const float *img, const float *tgt, int H, int W, Win win,
+                                                                 float C1, float C2, float *F, unsigned long long *acc)
 {
+    using Tile = FwdTile<WARPS, SEG>;
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
-    __shared__ float2 sxy[kFwdRowsH][kLTP];
-    __shared__ float2 hb01[kFwdRowsH][kLT + 1], hb23[kFwdRowsH][kLT + 1];
-    __shared__ float hb4[kFwdRowsH][kLT + 1];
-    __shared__ float red[2][kFwdWarps];
+    __shared__ float2 sxy[Tile::rows_h][kLTP];
+    __shared__ float2 hb01[Tile::rows_h][kLT + 1], hb23[Tile::rows_h][kLT + 1];
+    __shared__ float hb4[Tile::rows_h][kLT + 1];
+    __shared__ float red[2][WARPS];
     const int plane = blockIdx.z;
     float2 w[6];
     window_pairs(win, w);
     const float *x = img + (long long)plane * H * W;
     const float *y = tgt + (long long)plane * H * W;
-    const int ox = blockIdx.x * kLT, oy = blockIdx.y * kFwdRows;
+    const int ox = blockIdx.x * kLT, oy = blockIdx.y * Tile::rows;
     {
         // every load of the thread issued before the first store
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        float2 buf[kFwdStageRows][2];
+        float2 buf[Tile::stage_rows][2];
 #pragma unroll
-        for (int q = 0; q < kFwdStageRows; q++)
+        for (int q = 0; q < Tile::stage_rows; q++)
 #pragma unroll
             for (int h = 0; h < 2; h++) {
-                const int r = warp + kFwdWarps * q, c = lane + 32 * h;
+                const int r = warp + WARPS * q, c = lane + 32 * h;
                 const int gy = oy + r - kHalo, gx = ox + c - kHalo;
-                buf[q][h] = r < kFwdRowsH && c < kLTH ? make_float2(ld_zero(x, H, W, gy, gx), ld_zero(y, H, W, gy, gx))
+                buf[q][h] = r < Tile::rows_h && c < kLTH ? make_float2(ld_zero(x, H, W, gy, gx), ld_zero(y, H, W, gy, gx))
                                                  : make_float2(0.f, 0.f);
             }
 #pragma unroll
-        for (int q = 0; q < kFwdStageRows; q++)
+        for (int q = 0; q < Tile::stage_rows; q++)
 #pragma unroll
             for (int h = 0; h < 2; h++) {
-                const int r = warp + kFwdWarps * q, c = lane + 32 * h;
-                if (r < kFwdRowsH && c < kLTH) sxy[r][c] = buf[q][h];
+                const int r = warp + WARPS * q, c = lane + 32 * h;
+                if (r < Tile::rows_h && c < kLTH) sxy[r][c] = buf[q][h];
             }
     }
     __syncthreads();
-    // horizontal blur of (x, y), (x^2, y^2) and xy: 46 rows x (32 / kHSeg) segments,
+    // horizontal blur of (x, y), (x^2, y^2) and xy: the rows with the halo x (32 / kHSeg) segments,
     // consecutive threads on consecutive rows (no bank conflicts)
     // input by input: each input's products x^2, y^2 and xy are formed once and
     // added to the kHSeg outputs whose window holds it
-    for (int wi = threadIdx.x; wi < kFwdRowsH * (kLT / kHSeg); wi += kFwdThreads) {
-        const int r = wi % kFwdRowsH, c0 = (wi / kFwdRowsH) * kHSeg;
+    for (int wi = threadIdx.x; wi < Tile::rows_h * (kLT / kHSeg); wi += Tile::threads) {
+        const int r = wi % Tile::rows_h, c0 = (wi / Tile::rows_h) * kHSeg;
         float2 a01[kHSeg], a23[kHSeg];
         float a4[kHSeg];
 #pragma unroll
@@ -138,20 +140,20 @@ __global__ void __launch_bounds__(kFwdThreads, 4) ssim_fwd_kernel(const float *i
         for (int o = 0; o < kHSeg; o++) { hb01[r][c0 + o] = a01[o]; hb23[r][c0 + o] = a23[o]; hb4[r][c0 + o] = a4[o]; }
     }
     __syncthreads();
-    // vertical blur and the SSIM terms: 32 columns x kFwdWarps segments
+    // vertical blur and the SSIM terms: 32 columns x WARPS segments
     float ssum = 0.f, l1sum = 0.f;
     {
-        const int c = threadIdx.x % kLT, r0 = (threadIdx.x / kLT) * kFwdVSeg;
-        float2 m01[kFwdVSeg], m23[kFwdVSeg];
-        float m4[kFwdVSeg];
+        const int c = threadIdx.x % kLT, r0 = (threadIdx.x / kLT) * SEG;
+        float2 m01[SEG], m23[SEG];
+        float m4[SEG];
 #pragma unroll
-        for (int o = 0; o < kFwdVSeg; o++) { m01[o] = f2s(0.f); m23[o] = f2s(0.f); m4[o] = 0.f; }
+        for (int o = 0; o < SEG; o++) { m01[o] = f2s(0.f); m23[o] = f2s(0.f); m4[o] = 0.f; }
 #pragma unroll
-        for (int j = 0; j < kFwdVSeg + 10; j++) {
+        for (int j = 0; j < SEG + 10; j++) {
             const float2 v01 = hb01[r0 + j][c], v23 = hb23[r0 + j][c];
             const float v4 = hb4[r0 + j][c];
 #pragma unroll
-            for (int o = 0; o < kFwdVSeg; o++) {
+            for (int o = 0; o < SEG; o++) {
                 const int t = j - o;
                 if (t >= 0 && t < 11) {
                     const float2 wt = w[tap(t)];
@@ -162,7 +164,7 @@ __global__ void __launch_bounds__(kFwdThreads, 4) ssim_fwd_kernel(const float *i
             }
         }
 #pragma unroll
-        for (int o = 0; o < kFwdVSeg; o++) {
+        for (int o = 0; o < SEG; o++) {
             const int r = r0 + o;
             const int gy = oy + r, gx = ox + c;
             if (gy >= H || gx >= W) continue;
@@ -193,7 +195,7 @@ __global__ void __launch_bounds__(kFwdThreads, 4) ssim_fwd_kernel(const float *i
     __syncthreads();
     if (threadIdx.x == 0) {
         float a = 0.f, b = 0.f;
-        for (int q = 0; q < kFwdWarps; q++) { a += red[0][q]; b += red[1][q]; }
+        for (int q = 0; q < WARPS; q++) { a += red[0][q]; b += red[1][q]; }
         // the view's sums in 64-bit fixed point (24 fractional bits): integer
         // atomics add exactly, so the totals do not depend on block order
         const int view = blockIdx.z / 3;
@@ -331,13 +333,20 @@ cudaError_t launch_loss(gs_workspace *ws, cudaStream_t st, const float *img, con
     for (int k = 0; k < 11; k++) { g[k] = exp(-((k - 5) * (k - 5)) / (2.0 * 1.5 * 1.5)); sum += g[k]; }
     for (int k = 0; k < 6; k++) win.w[k] = (float)(g[k] / sum);
     const dim3 grid((W + kLT - 1) / kLT, (H + kLT - 1) / kLT, B * 3);
-    const dim3 fgrid(grid.x, (H + kFwdRows - 1) / kFwdRows, B * 3);
+    // 32 rows by eight warps while all such tiles are resident at once (four blocks per
+    // SM) and a tile's own latency is the time: the forward of 64 x 64 takes 7.8 us
+    // against 8.5 with 36 rows, of two views of 300 x 400 (780 tiles for 608 places) 14.7
+    // against 13.6; between 300 and 600 tiles the two are alike
+    const bool tall = (long long)grid.x * grid.y * grid.z > 4ll * ws->sm_count;
+    const int frows = tall ? FwdTile<6, 6>::rows : FwdTile<8, 4>::rows;
+    const int fthreads = tall ? FwdTile<6, 6>::threads : FwdTile<8, 4>::threads;
+    const dim3 fgrid(grid.x, (H + frows - 1) / frows, B * 3);
     float *maps = ws->loss_maps; // three planes per image plane
     unsigned long long *acc = reinterpret_cast<unsigned long long *>(ws->loss_partial); // [B][2]
     cudaError_t e = cudaMemsetAsync(acc, 0, 2 * (size_t)B * sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
     kt_begin(ws, GS_KT_SSIM_FWD, st);
-    launch_pdl(ssim_fwd_kernel, fgrid, kFwdThreads, 0, st, img, tgt, H, W, win, 0.01f * 0.01f, 0.03f * 0.03f, maps, acc);
+    launch_pdl(tall ? ssim_fwd_kernel<6, 6> : ssim_fwd_kernel<8, 4>, fgrid, fthreads, 0, st, img, tgt, H, W, win, 0.01f * 0.01f, 0.03f * 0.03f, maps, acc);
     kt_end(ws, GS_KT_SSIM_FWD, st);
     note_launch();
     kt_begin(ws, GS_KT_SSIM_BWD, st);

@@ -1,5 +1,5 @@
-"""The loss at image sizes around the edges of its tiles (32 columns; 36 rows in
-the forward, 32 in the adjoint), against the float64 oracle."""
+"""The loss at image sizes around the edges of its tiles (32 columns; 32 rows, or 36
+in the forward of many tiles), against the float64 oracle."""
 import numpy as np
 import pytest
 import torch
@@ -22,12 +22,14 @@ def _built():
 # any other size
 @pytest.mark.parametrize("views,h,w", [(1, 1, 1), (1, 1, 40), (1, 40, 1), (1, 5, 6), (2, 31, 31), (1, 32, 33), (1, 35, 32),
                                        (1, 36, 32), (3, 37, 33), (1, 41, 27), (1, 64, 64), (1, 71, 65), (1, 72, 31),
-                                       (2, 73, 96), (1, 108, 97)])
+                                       (2, 73, 96), (1, 108, 97),
+                                       # more tiles than are resident at once: the forward's 36 rows
+                                       (4, 71, 900), (4, 72, 897), (4, 73, 899), (7, 37, 900), (2, 109, 1500)])
 def test_sizes_around_the_tile_edges(views, h, w):
     rng = np.random.default_rng(1000 * h + w)
     x = rng.uniform(0, 1, (views, 3, h, w)).astype(np.float32)
     y = rng.uniform(0, 1, (views, 3, h, w)).astype(np.float32)
-    ws = B.Workspace(max_gaussians=1, max_records=1, max_instances=1, max_tiles=64, max_pixels=views * h * w)
+    ws = B.Workspace(max_gaussians=1, max_records=1, max_instances=1, max_tiles=64, max_cameras=1, max_pixels=views * h * w)
     xt, yt = torch.from_numpy(x).cuda(), torch.from_numpy(y).cuda()
     loss, dL = torch.zeros(1, device="cuda"), torch.empty_like(xt)
     ws.photometric_loss(xt, yt, 0.2, loss, dL)
