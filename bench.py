@@ -385,12 +385,12 @@ def bwd_roofline(fragments, composited, instances, pixels, kernel_ms, sm_mhz, pe
 #   view gate: per Gaussian its mean 12 B, level 1 B and mean drift 4 B; per
 #     candidate its log-scales 12 B and their drift 4 B read, its id 4 B and
 #     camera mask 8 B written
-#   binning, count pass: per record 18 B (tile count, rectangle, camera read,
-#     first instance written), per instance 4 B (its tile's count)
-#   binning, ranges, scatter and per-tile sort: per tile 20 B (count read,
-#     range and cursor written), per record 18 B (read again), per instance
-#     28 B (cursor, depth key read; key and record written; both read and the
-#     record written by the per-tile sort)
+#   binning, count pass: per record 14 B (first instance, rectangle, camera
+#     read), per instance 8 B (its tile's count, its rank written)
+#   binning, ranges, scatter and per-tile sort: per tile 20 B (count read and
+#     cleared, range and forward's maximum written), per record 18 B (the same
+#     and the depth key), per instance 24 B (rank read; key and record written;
+#     both read and the record written by the per-tile sort)
 #   slot reduction: per instance 36 B (its slot); per record 16 B of indices
 #     and 36 B of summed gradient written
 #   projection adjoint: per visible Gaussian 44 B of shape and opacity and
@@ -403,13 +403,13 @@ def bwd_roofline(fragments, composited, instances, pixels, kernel_ms, sm_mhz, pe
 #     read and written) and its 236 B gradient row
 HBM_KERNELS = {
     "gate_count_kernel": ("GS_KT_GATE", lambda c: 17 * c["n"] + 28 * c["n_candidates"]),
-    "bin_count": ("GS_KT_BIN_COUNT", lambda c: 18 * c["n_records"] + 4 * c["n_instances"]),
-    "bin_sort": ("GS_KT_BIN_SORT", lambda c: 20 * c["tiles"] + 18 * c["n_records"] + 28 * c["n_instances"]),
+    "bin_count": ("GS_KT_BIN_COUNT", lambda c: 14 * c["n_records"] + 8 * c["n_instances"]),
+    "bin_sort": ("GS_KT_BIN_SORT", lambda c: 20 * c["tiles"] + 18 * c["n_records"] + 24 * c["n_instances"]),
     "reduce_slots_kernel": ("GS_KT_REDUCE_SLOTS", lambda c: 36 * c["n_instances"] + 52 * c["n_records"]),
     "preprocess_bwd_kernel": ("GS_KT_PREPROCESS_BWD", lambda c: 472 * c["n_visible"] + 64 * c["n_records"]),
     "ssim_fwd_kernel": ("GS_KT_SSIM_FWD", lambda c: 20 * 3 * c["pixels"]),
     "ssim_bwd_kernel": ("GS_KT_SSIM_BWD", lambda c: 24 * 3 * c["pixels"]),
-    "lazy_list_vec_kernel (gradient step)": ("GS_KT_ADAM_GRAD", lambda c: (59 * 24 + 236) * c["n_visible"]),
+    "lazy_list_kernel (gradient step)": ("GS_KT_ADAM_GRAD", lambda c: (59 * 24 + 236) * c["n_visible"]),
 }
 
 

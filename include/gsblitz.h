@@ -3,8 +3,8 @@
  * Implements the per-iteration render of BlitzGS (arXiv 2605.13794) on one GPU:
  *   gs_preprocess  view gate (Sec. 3.3, Eq. 1-3) + EWA projection and SH colour
  *                  (App. A: "projected to screen-space ellipses", c_i(d) by SH)
- *   gs_bin_sort    tile/depth keys and a device radix sort (App. A: tile-based,
- *                  depth-ordered projected Gaussians)
+ *   gs_bin_sort    tile lists in depth order (App. A: tile-based, depth-ordered
+ *                  projected Gaussians)
  *   gs_render_fwd  front-to-back alpha compositing (App. A, Eq. for C(p), T_i)
  *   gs_render_bwd  its adjoint and the adjoint of the projection, plus the
  *                  scale regulariser of Eq. 5
@@ -221,7 +221,7 @@ int gs_workspace_destroy(gs_workspace *ws);
 /* Bytes of device memory a workspace with these capacities holds. */
 int64_t gs_workspace_bytes(const gs_capacity *cap);
 /* Execution tuning that leaves every result unchanged: keys ranked per block
- * by the radix passes of gs_bin_sort and gs_importance, 1024, 2048 or 4096;
+ * by the radix passes of gs_importance, 1024, 2048 or 4096;
  * 0 (the default) picks by the size of each sort (1024 up to 2^18 keys of
  * capacity, 2048 up to 2^20, 4096 above).  Applies to the calls made after it. */
 int gs_workspace_set_sort_chunk(gs_workspace *ws, int32_t keys_per_block);
@@ -251,7 +251,7 @@ int gs_upload_cameras(gs_workspace *ws, const gs_camera *cams, int32_t n_cams, c
 int gs_preprocess_uploaded(gs_workspace *ws, const gs_gaussians *g, const uint32_t *cull,
                            const gs_render_params *params, gs_stream stream);
 
-/* Tile keys, device radix sort by (camera, tile, depth, record), tile ranges. */
+/* Every tile's list of records in (depth, record) order, and the tile ranges. */
 int gs_bin_sort(gs_workspace *ws, gs_stream stream);
 
 /* Front-to-back compositing.  rgb_out: [sum over cameras of 3*H*W], camera c's
@@ -502,7 +502,7 @@ enum {
     GS_KT_IMPORTANCE = 2,      /* the importance sweep's rasteriser */
     GS_KT_GATE = 3,            /* the view gate's pass over every Gaussian (gs_preprocess) */
     GS_KT_PROJECT = 4,         /* the projection of the gate's candidates (gs_preprocess) */
-    GS_KT_BIN_COUNT = 5,       /* gs_bin_sort: each record's first instance and the tile counts */
+    GS_KT_BIN_COUNT = 5,       /* gs_bin_sort: the tile counts and each instance's rank in its tile */
     GS_KT_BIN_SORT = 6,        /* gs_bin_sort: tile ranges, scatter by tile and the per-tile depth sort */
     GS_KT_REDUCE_SLOTS = 7,    /* the per-record sum of the adjoint's gradient slots */
     GS_KT_PREPROCESS_BWD = 8,  /* the projection adjoint (per Gaussian) */

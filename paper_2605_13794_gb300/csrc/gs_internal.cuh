@@ -91,7 +91,6 @@ __device__ __forceinline__ void slot_grads_from_moments(float (&g)[kSlotFloats],
 // Error sites recorded next to the error word (which kernel gave up).
 enum ErrorSite {
     kSitePreprocess = 1, kSiteEmit = 2 /* binning */, kSiteRadix = 3, kSiteSelect = 4, kSiteScanF64 = 5, kSiteModel = 6,
-    kSiteRender = 7,
 };
 
 // Device counters of one workspace.

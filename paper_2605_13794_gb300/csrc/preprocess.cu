@@ -817,8 +817,8 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(GaussPtrs g, PreO
 // and instances known -- the records, which consecutive threads write to
 // consecutive places.  A thread per candidate waited for the candidate of the most
 // cameras, stored its records strided and read the first colours only after the
-// look-back: 24 mixed views of the 4M city took 282 us of 2531 and the whole now
-// takes 2403, eight 1600 x 1200 views of 8M 7170 and 7062, the importance pass of
+// look-back: it took 282 us for 24 mixed views of the 4M city and this takes 149, the
+// whole pass 2531 and 2403, eight 1600 x 1200 views of 8M 7170 and 7062, the importance pass of
 // eight views 1000 and 970; two views of 20k Gaussians stay at 263.
 // kViewsBlocks: 64 registers; with seven blocks (72) the 24 views take 2406, six 2413.
 constexpr int kViewsBlocks = 8; // blocks per SM
