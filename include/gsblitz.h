@@ -314,7 +314,10 @@ int gs_adam_step_compact(gs_workspace *ws, const gs_gaussians *g, const gs_gauss
  *     first step) when enabling; drift: [2][n] float, zeroed by the caller (per
  *     Gaussian, bounds on how far its mean and its largest log-scale can still
  *     move, which widen the view gate);
- *   max_steps: steps the workspace keeps coefficients for (40 bytes each);
+ *   max_steps: steps the workspace keeps coefficients for (40 bytes each); a
+ *     step past it is refused with GS_ERR_CAPACITY (by the call if it names the
+ *     step, by the device error word if it takes the device counter's) and
+ *     changes neither the counter nor any parameter or moment;
  *   every moment array 16-byte aligned (as the parameter arrays);
  *   needs beta1 < sqrt(beta2).  Allocates the step history (once, here). */
 int gs_adam_lazy_enable(gs_workspace *ws, const gs_gaussian_grads *m, const gs_gaussian_grads *v, int32_t *last_step,

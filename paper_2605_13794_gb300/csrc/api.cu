@@ -119,7 +119,7 @@ Offsets plan(const gs_capacity &c)
     o.red_partial = L.take<float>(o.red_words);
     o.ctr = L.take<gs::DevCounters>(1);
     o.d_cams = L.take<gs::CamTable>(1);
-    o.d_adam_step = L.take<int>(1);
+    o.d_adam_step = L.take<int>(2);
     o.d_adam_coef = L.take<float>(2 * GS_MAX_ADAM_GROUPS);
     const size_t NM = (c.flags & GS_CAP_MODEL_OPS) ? N : 0; // model-level scratch
     o.mkey0 = L.take<uint32_t>(NM);
@@ -329,7 +329,7 @@ int gs_workspace_create(const gs_capacity *cap, gs_workspace **out)
     // zero between binnings: every binning leaves them so
     if (e == cudaSuccess) e = cudaMemset(ws->bin_lb, 0, o.bin_lb_words * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemset(ws->tile_cnt, 0, (size_t)cap->max_tiles * sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMemset(ws->d_adam_step, 0, sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(ws->d_adam_step, 0, 2 * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(ws->mctr, 0, sizeof(gs::DevCounters));
     if (e == cudaSuccess) e = cudaMallocHost(&ws->h_stage, gs_workspace::kStageSlots * sizeof(gs::CamTable));
     for (int k = 0; e == cudaSuccess && k < gs_workspace::kStageSlots; k++) {
@@ -639,6 +639,9 @@ int gs_adam_step_compact(gs_workspace *ws, const gs_gaussians *g, const gs_gauss
         (m->mean != ws->lazy.m.mean || v->mean != ws->lazy.v.mean || beta1 != ws->lazy.b1 || beta2 != ws->lazy.b2 ||
          eps != ws->lazy.eps))
         return fail(GS_ERR_INVALID_ARG, "gs_adam_step_compact: moments and betas must be those of gs_adam_lazy_enable");
+    if (ws->lazy.enabled && step > ws->lazy.max_steps)
+        return fail(GS_ERR_CAPACITY, "gs_adam_step_compact: step %d exceeds the max_steps %d of gs_adam_lazy_enable", step,
+                    ws->lazy.max_steps);
     gs_gaussian_grads param;
     param.mean = const_cast<float *>(g->mean);
     param.log_scale = const_cast<float *>(g->log_scale);

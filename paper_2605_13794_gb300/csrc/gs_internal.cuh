@@ -421,7 +421,8 @@ struct gs_workspace {
     unsigned long long *mlb;     // single-value look-back, [N / 256 + 3]
     uint32_t *mhist;             // [4][256]
     gs::DevCounters *mctr;       // item count (n_records) and errors of the model-level calls
-    int *d_adam_step;      // device Adam step counter (graph-replayable optimizer step)
+    int *d_adam_step;      // device Adam step counter (graph-replayable optimizer step); then 1 if the last
+                           // step was refused because its coefficients have no row in lazy.hist
     // deferred zero-gradient Adam steps (gs_adam_lazy_enable): a Gaussian's p, m,
     // v are brought to the current step only when it is next used
     struct {

@@ -553,13 +553,21 @@ struct AdamCoefArgs {
 // Step number and bias-corrected coefficients on the device, so a captured
 // optimizer step advances its own counter on every replay.  With deferred
 // steps enabled the coefficients of every step are also kept (hist), so a
-// Gaussian brought up to date later replays exactly the steps it missed.
+// Gaussian brought up to date later replays exactly the steps it missed; a step
+// that hist has no row for is refused: the counter stays, and d_step[1] tells
+// the update kernel to take no step.
 __global__ void adam_coef_kernel(AdamCoefArgs a, int *d_step, float *coef, float *hist, int max_steps,
                                  DevCounters *ctr)
 {
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
     if (threadIdx.x != 0) return;
     const int t = a.step > 0 ? a.step : *d_step + 1;
+    const bool refused = hist && t > max_steps;
+    d_step[1] = refused;
+    if (refused) {
+        set_error(ctr, GS_ERR_CAPACITY, kSiteModel);
+        return;
+    }
     *d_step = t;
     const double c1 = 1.0 - powi((double)a.b1, t), c2 = 1.0 - powi((double)a.b2, t);
     for (int k = 0; k < 5; k++) {
@@ -567,10 +575,6 @@ __global__ void adam_coef_kernel(AdamCoefArgs a, int *d_step, float *coef, float
         coef[GS_MAX_ADAM_GROUPS + k] = (float)(1.0 / sqrt(c2));
     }
     if (hist) {
-        if (t > max_steps) {
-            set_error(ctr, GS_ERR_CAPACITY, kSiteModel);
-            return;
-        }
         for (int k = 0; k < 5; k++) {
             hist[10 * t + k] = coef[k];
             hist[10 * t + 5 + k] = coef[GS_MAX_ADAM_GROUPS + k];
@@ -603,9 +607,13 @@ struct LazyArgs {
     long long n;       // Gaussians
     const float *hist;
     const int *d_step;
+    int max_steps;     // rows of hist after row 0
     float b1, b2, eps, drift_factor;
 };
 
+// The step to bring Gaussians to: the device counter, but never past the history
+// (a counter that an earlier, longer history left).
+__device__ __forceinline__ int lazy_step(const LazyArgs &a) { return min(*a.d_step, a.max_steps); }
 
 __device__ __forceinline__ int group_len(int k) { return k == 4 ? 48 : k == 3 ? 1 : k == 2 ? 4 : 3; }
 
@@ -682,7 +690,7 @@ __device__ __forceinline__ void lazy_all_group(const LazyArgs &a, int k, long lo
 __global__ void __launch_bounds__(256) lazy_all_elem_kernel(LazyArgs a, long long n)
 {
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
-    const int t = *a.d_step;
+    const int t = lazy_step(a);
     lazy_all_group<3>(a, 0, n, t);   // mean
     lazy_all_group<3>(a, 1, n, t);   // log-scale
     lazy_all_group<4>(a, 2, n, t);   // quaternion
@@ -719,7 +727,8 @@ constexpr int kLazyGradItems = 8;
 template <int MODE> __global__ void __launch_bounds__(256, 4) lazy_list_kernel(LazyArgs a, LazyItems it)
 {
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
-    const int t = *a.d_step;
+    if (MODE == kLazyGrad && a.d_step[1]) return; // the step was refused
+    const int t = lazy_step(a);
     const unsigned long long total = MODE == kLazyGrad ? it.ctr->n_records : it.ctr->n_candidates;
     const int lane = threadIdx.x & 31, u = lane & 15;
     const int k = u < 12 ? 4 : u == 12 ? 2 : u == 13 ? 0 : u == 14 ? 1 : 3;
@@ -809,7 +818,7 @@ template <int MODE> __global__ void __launch_bounds__(256, 4) lazy_list_kernel(L
 __global__ void __launch_bounds__(256) lazy_fin_kernel(LazyArgs a)
 {
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
-    const int t = *a.d_step;
+    const int t = lazy_step(a);
     for (long long i = blockIdx.x * 256ll + threadIdx.x; i < a.n; i += gridDim.x * 256ll) {
         if (a.last[i] >= t) continue;
         a.last[i] = t;
@@ -831,6 +840,7 @@ static LazyArgs lazy_args(gs_workspace *ws, const gs_gaussian_grads &param, long
     a.drift = ws->lazy.drift;
     a.hist = ws->lazy.hist;
     a.d_step = ws->d_adam_step;
+    a.max_steps = ws->lazy.max_steps;
     a.b1 = ws->lazy.b1; a.b2 = ws->lazy.b2; a.eps = ws->lazy.eps; a.drift_factor = ws->lazy.drift_factor;
     return a;
 }
