@@ -360,10 +360,11 @@ __device__ __forceinline__ bool cull_bit(const PreOut &o, int c, long long i)
 }
 
 // The cameras of the call, copied from the device table into shared memory
-// once per block (every Gaussian reads them).
-__device__ __forceinline__ void stage_cameras(const CamTable &ct, CamInfo *s_cams)
+// once per block (every Gaussian reads them).  At most the N there is room for: a
+// kernel of one camera in a captured graph may meet a table of more.
+template <int N> __device__ __forceinline__ void stage_cameras(const CamTable &ct, CamInfo (&s_cams)[N])
 {
-    const int words = ct.n * (int)(sizeof(CamInfo) / sizeof(int));
+    const int words = min(ct.n, N) * (int)(sizeof(CamInfo) / sizeof(int));
     const int *src = reinterpret_cast<const int *>(ct.c);
     int *dst = reinterpret_cast<int *>(s_cams);
     for (int w = threadIdx.x; w < words; w += blockDim.x) dst[w] = src[w];
