@@ -324,7 +324,7 @@ struct PreOut {
     uint8_t *clampm;
     uint32_t *cand_g;
     unsigned long long *cand_mask;
-    uint32_t *gate_g;              // [N] block-strided candidates of the gate's first pass
+    uint32_t *gate_g;              // [N] the gate's candidates, each chunk's at the start of its own range
     unsigned long long *gate_mask; // [N]
     const float *drift;            // [2][N] drift bounds (mean, log-scale) of deferred Adam steps, or NULL
     uint32_t *inst_off, *chunk_rec;
@@ -340,18 +340,14 @@ struct PreOut {
 
 struct GaussLoad {
     float m[3], ls[3], q[4];
-    float smax;
-    bool have_shape;
 };
 
-__device__ __forceinline__ void load_shape(const GaussPtrs &g, long long i, GaussLoad &L)
+__device__ __forceinline__ void load_gauss(const GaussPtrs &g, long long i, GaussLoad &L)
 {
-    if (L.have_shape) return;
+    L.m[0] = g.mean[3 * i]; L.m[1] = g.mean[3 * i + 1]; L.m[2] = g.mean[3 * i + 2];
     L.ls[0] = g.log_scale[3 * i]; L.ls[1] = g.log_scale[3 * i + 1]; L.ls[2] = g.log_scale[3 * i + 2];
     const float4 q = *reinterpret_cast<const float4 *>(g.quat + 4 * i); // 16-byte aligned rows
     L.q[0] = q.x; L.q[1] = q.y; L.q[2] = q.z; L.q[3] = q.w;
-    L.smax = expf(fmaxf(L.ls[0], fmaxf(L.ls[1], L.ls[2])));
-    L.have_shape = true;
 }
 
 __device__ __forceinline__ bool cull_bit(const PreOut &o, int c, long long i)
@@ -707,11 +703,10 @@ __device__ __forceinline__ void store_record(const PreOut &o, unsigned long long
     o.clampm[r] = q.clm;
 }
 
-// kOneCam: a candidate has at most one record, which is computed (colour
-// included, from the projection that decided it) before the block's scan and
-// look-back, so the look-back of one warp does not leave the others idle in
-// front of the colour's loads.  Blocks of kProjThreads take chunks of as many
-// candidates.
+// One camera: a candidate has at most one record, whose colour is read before the
+// block's look-back is resolved, so the look-back of one warp does not leave the
+// others idle in front of the colour's loads.  Blocks of kProjThreads take chunks
+// of as many candidates.
 constexpr int kProjThreads = 128;
 __global__ void __launch_bounds__(kProjThreads) project_kernel(GaussPtrs g, PreOut o, const CamTable *__restrict__ ctp,
                                                                RenderConsts rc)
@@ -719,7 +714,7 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(GaussPtrs g, PreO
     constexpr int kNW = kProjThreads / 32;
     griddep_wait(); // programmatic dependent launch: the previous kernel is complete
     const CamTable &ct = *ctp;
-    __shared__ CamInfo s_cams[GS_MAX_CAMERAS];
+    __shared__ CamInfo s_cam[1];
     __shared__ float s_thr2[kMaxLod + 1];
     __shared__ unsigned s_bid;
     __shared__ unsigned long long s_warp[kNW];
@@ -730,7 +725,8 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(GaussPtrs g, PreO
 #pragma unroll
         for (int l = 0; l <= kMaxLod; l++) s_thr2[l] = rc.lod_thr2[l];
     }
-    stage_cameras(ct, s_cams);
+    stage_cameras(ct, s_cam);
+    const CamInfo &cam = s_cam[0];
     // persistent blocks: each takes the next chunk of candidates (tickets in
     // order, so every look-back waits only on chunks already being processed)
     for (;;) {
@@ -740,52 +736,37 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(GaussPtrs g, PreO
     if ((unsigned long long)bid * kProjThreads >= ncand) return;
     const unsigned long long j = (unsigned long long)bid * kProjThreads + threadIdx.x;
     GaussLoad L;
-    L.have_shape = false;
     long long i = 0;
-    unsigned long long act = 0, tiles = 0; // active cameras, tiles of their records
+    bool act = false;
+    unsigned long long tiles = 0; // of the candidate's record
     float op = 0.f;
-    Proj p_one; // one camera: the projection of the active record
+    Proj p;
     if (j < ncand) {
         i = o.cand_g[j];
-        const unsigned long long cm = 1ull;
-        L.m[0] = g.mean[3 * i]; L.m[1] = g.mean[3 * i + 1]; L.m[2] = g.mean[3 * i + 2];
-        load_shape(g, i, L);
+        load_gauss(g, i, L);
         const float ol = g.opacity_logit[i];
         const int lod = (rc.lod_enable && g.lod) ? (int)g.lod[i] : 0;
-        for (unsigned long long mm = cm; mm; mm &= mm - 1) {
-            const int c = __ffsll((long long)mm) - 1;
-            // the exact LOD decision (the gate's is widened for Gaussians with deferred steps)
-            if (!lod_pass(L.m, lod, s_cams[c], rc, s_thr2)) continue;
+        // the exact LOD decision (the gate's is widened for Gaussians with deferred steps)
+        if (lod_pass(L.m, lod, cam, rc, s_thr2)) {
             DF td[3];
-            camera_point_df(L.m, s_cams[c], td);
-            if (!(td[2].hi > rc.znear)) continue;
-            Proj p;
-            if (project_gaussian(L.ls, L.q, td, s_cams[c], tw, th, rc, p)) {
-                act |= 1ull << c;
-                tiles += (unsigned)((p.x1 - p.x0) * (p.y1 - p.y0));
-                p_one = p;
-            }
+            camera_point_df(L.m, cam, td);
+            act = td[2].hi > rc.znear && project_gaussian(L.ls, L.q, td, cam, tw, th, rc, p);
+            if (act) tiles = (unsigned)((p.x1 - p.x0) * (p.y1 - p.y0));
         }
         op = 1.f / (1.f + expf(-ol));
     }
-    const unsigned long long cnt = __popcll(act);
-    // GS_CULL_MARK: records of the cameras whose Cull bit is set are kept and marked
-    unsigned long long marked = 0;
-    if (rc.cull_enable == GS_CULL_MARK)
-        for (unsigned long long mm = act; mm; mm &= mm - 1) {
-            const int c = __ffsll((long long)mm) - 1;
-            if (cull_bit(o, c, i)) marked |= 1ull << c;
-        }
+    // GS_CULL_MARK: a record whose Cull bit is set is kept and marked
+    const bool marked = act && rc.cull_enable == GS_CULL_MARK && cull_bit(o, 0, i);
     unsigned long long total, itotal;
-    const unsigned long long excl = block_exclusive_scan<kNW, unsigned long long>(cnt, s_warp, total);
+    const unsigned long long excl = block_exclusive_scan<kNW, unsigned long long>(act, s_warp, total);
     const unsigned long long iexcl = block_exclusive_scan<kNW, unsigned long long>(tiles, s_warp, itotal);
-    const int tvis = __syncthreads_count((act & ~marked) != 0);
+    const int tvis = __syncthreads_count(act && !marked);
     // the chunk's counts are published before the colours are read, so that no
     // later chunk's look-back waits for them
     if (threadIdx.x == 0) lookback_publish(o.lb_status + 1, bid, total);
     if (threadIdx.x == 32) lookback_publish(o.lb_inst, bid, itotal);
     RecOut one;
-    if (act) one = make_record(g, i, L, op, s_cams[0], p_one, rc, marked & 1ull);
+    if (act) one = make_record(g, i, L, op, cam, p, rc, marked);
     if (threadIdx.x < 32) {
         const unsigned long long b = lookback_resolve(o.lb_status + 1, bid, total, o.ctr, kSitePreprocess);
         if (threadIdx.x == 0) {
@@ -800,7 +781,7 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(GaussPtrs g, PreO
     const unsigned long long base = s_base + excl, ibase = s_ibase + iexcl;
     if (j == ncand - 1) {
         o.ctr->inst_total = ibase + tiles;
-        const unsigned long long end = base + cnt;
+        const unsigned long long end = base + act;
         o.ctr->records_needed = end;
         o.ctr->n_records = end < (unsigned long long)o.max_records ? end : o.max_records;
     }
@@ -879,9 +860,7 @@ __global__ void __launch_bounds__(kProjThreads, kViewsBlocks) project_views_kern
             const int k = pair_of(s_mask, q, c);
             const long long i = s_g[k];
             GaussLoad L;
-            L.have_shape = false;
-            L.m[0] = g.mean[3 * i]; L.m[1] = g.mean[3 * i + 1]; L.m[2] = g.mean[3 * i + 2];
-            load_shape(g, i, L);
+            load_gauss(g, i, L);
             const int lod = (rc.lod_enable && g.lod) ? (int)g.lod[i] : 0;
             // the exact LOD decision (the gate's is widened for Gaussians with deferred steps)
             if (!lod_pass(L.m, lod, s_cams[c], rc, s_thr2)) continue;
@@ -913,9 +892,7 @@ __global__ void __launch_bounds__(kProjThreads, kViewsBlocks) project_views_kern
                 k = pair_of(s_act, q, c);
                 const long long i = s_g[k];
                 GaussLoad L;
-                L.have_shape = false;
-                L.m[0] = g.mean[3 * i]; L.m[1] = g.mean[3 * i + 1]; L.m[2] = g.mean[3 * i + 2];
-                load_shape(g, i, L);
+                load_gauss(g, i, L);
                 const float op = 1.f / (1.f + expf(-g.opacity_logit[i]));
                 DF td[3];
                 camera_point_df(L.m, s_cams[c], td);
