@@ -328,8 +328,8 @@ template <int E> __device__ __forceinline__ void warp_sort_regs(unsigned (&x)[E]
 // that place, which fetches the key from its copy in shared memory (stage, 32 E
 // of the warp's own).  Two keys that agree in those depth bits (equal depths,
 // above all) are in no order: then the 64-bit network sorts the list.
-// kWarpSort is 256: with 128, the lists of 129 to 256 entries go to the block and
-// the importance pass of eight views takes 1018 us for 1015.
+// kWarpSort is 256: with 128, the lists of 129 to 256 entries go to the block, which
+// makes no difference beyond the repeats' (importance pass of eight views).
 template <int E>
 __device__ __forceinline__ void sort_keys(const uint2 *p, uint32_t n, unsigned long long *stage,
                                           unsigned long long (&y)[E])

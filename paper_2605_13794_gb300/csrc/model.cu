@@ -264,7 +264,8 @@ __device__ __forceinline__ void copy_rows(const float *__restrict__ src, float *
 // copying its 177 floats one after another, as the list kernel once did, touched
 // a sector per float: the mass cut and compaction of 3M Gaussians with moments
 // took 2.52 ms and takes 0.98, the density control of 1.5M 2.32 and 0.67 (array by
-// array over the whole model, 62 registers: 1.14 and 0.82).  (A list entry left unset by a look-back that gave up is
+// array over the whole model, 62 registers: 1.14 and 0.82; the 32 registers of eight
+// blocks per SM spill 48 B).  (A list entry left unset by a look-back that gave up is
 // not followed: i < n.)
 template <bool VEC> __global__ void __launch_bounds__(256, 8) model_rows_kernel(ScatterArgs a)
 {

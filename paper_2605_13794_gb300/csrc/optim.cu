@@ -633,7 +633,7 @@ __device__ __forceinline__ int group_len(int k) { return k == 4 ? 48 : k == 3 ? 
 // a fixed point of the zero-gradient step (m and v stay +0, p moves by
 // (-lr m) / (sqrt(v) ibc2 + eps) = -0), so its replay is skipped and, without
 // a gradient step, it is not written at all.
-enum LazyMode { kLazyAll = 0, kLazyCandidates = 1, kLazyGrad = 2 };
+enum LazyMode { kLazyCandidates = 1, kLazyGrad = 2 };
 
 struct LazyItems {
     const uint32_t *list;      // Gaussian of each item: the gate's candidates, or each record's (a Gaussian's contiguous)

@@ -802,7 +802,8 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(GaussPtrs g, PreO
 // look-back: it took 282 us for 24 mixed views of the 4M city and this takes 149, the
 // whole pass 2531 and 2403, eight 1600 x 1200 views of 8M 7170 and 7062, the importance pass of
 // eight views 1000 and 970; two views of 20k Gaussians stay at 263.
-// kViewsBlocks: 64 registers; with seven blocks (72) the 24 views take 2406, six 2413.
+// kViewsBlocks: 64 registers with 32 B spilled; seven blocks (72) or six are alike within
+// what the repeats differ by.
 constexpr int kViewsBlocks = 8; // blocks per SM
 __global__ void __launch_bounds__(kProjThreads, kViewsBlocks) project_views_kernel(GaussPtrs g, PreOut o,
                                                                      const CamTable *__restrict__ ctp, RenderConsts rc)

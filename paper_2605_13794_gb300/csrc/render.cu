@@ -3,9 +3,10 @@
 // (Sec. 3.2, Fig. 2).
 //
 // One block per tile; each warp owns an 8 x 8 pixel square of it (lane l the
-// horizontal pixel pair (2 (l % 4), l / 4), packed FP32x2) and walks the
-// tile's depth-ordered list on its own, staging each batch of 32 entries
-// itself and visiting only the entries that can reach alpha_min in its square.
+// horizontal pixel pair (2 (l % 4), l / 4), packed FP32x2).  The block stages the
+// tile's depth-ordered list in rounds, an entry per thread, and each warp visits
+// those entries of a round that can reach alpha_min in its square (the adjoint:
+// those that composited there).
 // Per-Gaussian quantities are warp reductions (recursive halving for the
 // adjoint's nine values), then the warps' partials summed in warp order,
 // rather than per-pixel global atomics.  The backward and the importance
@@ -73,8 +74,8 @@ __device__ __forceinline__ float2 pair_alpha(float2 p, float o, float amax, floa
 // fails can reach alpha_min in them; it always fails when o is below alpha_min.
 // A warp skips an entry that fails: it composites nowhere in the warp, so
 // skipping it changes nothing.  (The bounding box of the ellipse and a looser
-// bound of q, before, took as many instructions and dropped fewer: the eight-view
-// training step of 8M Gaussians 7.68 ms with them, 7.61 with this test.)
+// bound of q, before, took as many instructions and dropped fewer entries; the
+// whole passes are alike within what their repeats differ by.)
 struct SquareTest {
     float A, k, D, tau, slope, u, v;
     __device__ __forceinline__ SquareTest(float4 r0, float D_, float o, float alpha_min, float u_, float v_)
@@ -157,12 +158,12 @@ __device__ __forceinline__ unsigned long long slot_of(const uint32_t *inst_off, 
 
 // ---- warp squares ------------------------------------------------------------
 //
-// The forward and the adjoint give each warp an 8 x 8 pixel square of the
-// tile: lane l holds the horizontal pixel pair (2 (l % 4), l / 4) of it, as
-// FP32x2, and the warp walks the tile's list on its own.  The warp stages each
-// batch of 32 entries itself (lane i the i-th), the staging lane tests its
-// entry's alpha footprint against the square (square_visit), and one ballot gives the entries the
-// warp visits; an entry whose box misses the square composites nowhere in it.
+// Every walk gives each warp an 8 x 8 pixel square of the tile: lane l holds the
+// horizontal pixel pair (2 (l % 4), l / 4) of it, as FP32x2.  A batch is 32
+// consecutive entries of the tile's list, staged by one warp for the whole block
+// (lane i the i-th); the staging lane tests its entry against every square
+// (SquareTest), and one ballot per square gives the entries of the batch that its
+// warp visits.
 
 template <int TW, int TH> struct SquareShape {
     static_assert(TW % 8 == 0 && TH % 8 == 0, "the tile splits into 8 x 8 pixel squares");
@@ -172,10 +173,11 @@ template <int TW, int TH> struct SquareShape {
     // the adjoint's register budget: at least six resident blocks of 128 threads per
     // SM, which ptxas meets with 64 registers (so eight fit); on the 16 x 16 tile
     // 10-15 % faster than both its own choice (86 registers, five blocks) and tighter
-    // budgets (56-57 registers)
+    // budgets (56-57 registers); both measured when each warp staged for itself
     static constexpr int bwd_min_blocks = 768 / threads;
     // the importance walk's: eight blocks of 128 threads (64 registers; the fused walk
-    // with the training image measured 8 % faster than with the compiler's 60)
+    // with the training image measured 8 % faster than with the compiler's 60, when each
+    // warp staged for itself)
     static constexpr int imp_min_blocks = 1024 / threads;
 };
 
@@ -255,6 +257,11 @@ __device__ __forceinline__ void put_visits(uint32_t *visits, int start, int b, i
 // T_min), which it asks once per batch: a vote after every entry cost more than
 // the entries it saved (24 mixed views, whole pass: 2.84 ms with it, 2.79
 // without), as did a vote to skip the entries that reach no live pixel (3.06).
+// Where every pixel stops within the first entries of a long list the walk alone is
+// slower than with batches staged per warp, by the round staged in vain (200k opaque
+// Gaussians of 45M instances at 720p: 37 and 54 us, their binning 7.8 and 4.5 ms);
+// asking before a round is staged whether any warp goes on does not help, the warps
+// of a tile finish together, and costs the other scenes 2 %.
 
 // VISITS: note the entries that composite in each square for the adjoint (not in
 // a forward-only workspace: the bookkeeping costs the walk 6 %).
@@ -644,7 +651,8 @@ cudaError_t launch_render_bwd(gs_workspace *ws, cudaStream_t st, const float *dL
 // the image, T and n_contrib equal render_fwd_kernel's and the slots this
 // kernel's alone, bit for bit.  (Warps staging for themselves and meeting at
 // arrival counters took 1.15 ms for the sweep of eight 1080p views of 3M
-// Gaussians, whole pass, this 1.04; the single-view training step 773 and 756 us.)
+// Gaussians, whole pass, this 1.04.  The fused walk of the 5M view is no faster than
+// it was, 148 and 147 us: the rounds pay for the visits that it notes besides.)
 
 struct ImpArgs {
     const uint2 *ranges;
